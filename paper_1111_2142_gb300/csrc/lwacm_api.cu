@@ -232,7 +232,7 @@ bool choose_kernel(lwacm_ctx *c) {
     static const char *hname[2][2] = {{"half_d3q19_tma", "half_d3q19_tma+scalar_rows"},
                                       {"half_d3q19_tma+nu_p_sum", "half_d3q19_tma+nu_p_sum+scalar_rows"}};
     c->kname = c->kernel == 5   ? hname[p.sdelta != 0.f ? 1 : 0][c->scalar_rows ? 1 : 0]
-               : c->kernel == 6 ? sname[c->batch_shape >= 0 && c->batch_shape < 7 ? c->batch_shape : 0]
+               : c->kernel == 6 ? (dev && c->batch_shape == 0 ? "tiles2d_d2q9_rows" : sname[c->batch_shape < 7 ? c->batch_shape : 0])
                                 : gname[c->Q == 19 ? 1 : 0];
     return ok;
 }
@@ -292,8 +292,8 @@ cudaError_t step_between(lwacm_ctx *c, const void *in, void *out, cudaStream_t s
     if (c->kernel == 5 && p.sdelta != 0.f) e = launch_nup_sum(c->storage, in, p.nup_p, p, st);
     if (e != cudaSuccess) return e;
     e = c->kernel == 5               ? launch_step_half(c->Q, c->storage, in, out, pf, st)
-                    : c->kernel == 6 ? launch_step_tiles2d(c->Q, c->storage, c->batch_shape > 0 ? c->batch_shape : 2,
-                                                           in, out, p, st)
+                    : c->kernel == 6 && c->batch_shape == 0 ? launch_step_rows2d(c->storage, in, out, p, st)
+                    : c->kernel == 6 ? launch_step_tiles2d(c->Q, c->storage, c->batch_shape, in, out, p, st)
                                      : launch_step_generic(c->Q, c->storage, in, out, p, st);
     if (e != cudaSuccess) return e;
     // the 2D-tile kernel applies the wall rule itself; the half-row kernel the x-face
@@ -428,7 +428,7 @@ std::vector<Cand> tune_candidates(const lwacm_ctx *c) {
         const int ks[2] = {5, 1};
         for (int k : ks) v.push_back(Cand{k, 0, 0});
         if (c->Q == 9)
-            for (int k = 1; k < batch_shapes(); ++k) v.push_back(Cand{6, k, 0});
+            for (int k = 0; k < batch_shapes(); ++k) v.push_back(Cand{6, k, 0});
     }
     return v;
 }
