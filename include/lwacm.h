@@ -100,7 +100,8 @@ enum {
                               and forcing applied in the kernel; omega_p and the
                               bulk-viscosity variant (alone or together) on periodic
                               domains; not the scalar; tile shape from
-                              LWACM_OPT_BATCH_TILE, 30x14 when 0). The automatic choice
+                              LWACM_OPT_BATCH_TILE; 0: strips of columns marched along
+                              y by warps). The automatic choice
                               takes 5, else 6, else 1. */
     LWACM_OPT_BATCH_MODE = 10, /* batched contexts: 0 = one launch per step, replayed
                                   from CUDA graphs (default); 1 = one persistent
@@ -114,8 +115,9 @@ enum {
                                      acceleration field (lwacm_set_force_field); only
                                      before lwacm_bind; single-domain contexts only */
     LWACM_OPT_BATCH_TILE = 13,    /* how domains are cut into CTA tiles. Batched contexts:
-                                     0 (default) = runs of 256 consecutive nodes, one
-                                     thread per node, every lattice; 1..6 = 2D tiles of
+                                     0 (default) = D2Q9: strips of 30 or 60 columns, each
+                                     updated by a warp that marches along y; D3Q19: runs
+                                     of 256 consecutive nodes; 1..6 = 2D tiles of
                                      30x6, 30x14, 62x6, 30x30, 62x14, 126x6 nodes, D2Q9
                                      only (LWACM_E_UNSUPPORTED otherwise), with the link
                                      values computed once per node and exchanged in

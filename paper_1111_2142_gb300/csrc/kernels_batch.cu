@@ -1,14 +1,21 @@
 // Batched update of many independent periodic domains of different sizes and
 // viscosities, packed one after the other in the same field arrays.
 //
-// The domains are cut into tiles of 256 consecutive nodes (a tile never spans two
+// D2Q9 domains are cut into strips of columns and runs of rows, each updated by a warp
+// that marches along y (rows2.cuh), from a table of items that holds what a warp needs of
+// its domain. 256 domains of 32 to 512 nodes a side (seed 1 of the benchmark): 37 us a
+// step, 187 GLUPS, against 118 us with one thread a node gathering from global memory and
+// 65 us in 2D tiles; bound by the latency of the last wave of items and the part of the
+// state that L2 does not hold.
+//
+// D3Q19 domains are cut into tiles of 256 consecutive nodes (a tile never spans two
 // domains); a CTA walks the tile list with a grid stride, one node per thread,
 // and updates it with the per-node moment form of Eq. ACM2.0 (node_update.cuh)
 // using its domain's (nx, ny, nz, nu).
 //
-//   k_batch_step        one launch = one step of every domain (the host replays
+//   k_batch_rows, k_batch_step  one launch = one step of every domain (the host replays
 //                       the steps from captured CUDA graphs);
-//   k_batch_persistent  one cooperative launch runs all the steps: the CTAs meet
+//   k_batch_*persistent one cooperative launch runs all the steps: the CTAs meet
 //                       at a grid-wide barrier between steps. The barrier spins a
 //                       bounded number of times; a CTA that gives up sets the
 //                       device error word to 2 and returns, so a missing arrival
@@ -27,6 +34,7 @@
 #include "launch.h"
 #include "lwacm_core.cuh"
 #include "node_update.cuh"
+#include "rows2.cuh"
 
 namespace lwacm {
 namespace {
@@ -296,6 +304,29 @@ __global__ void __launch_bounds__((TW + 2) * (TH + 2)) k_batch_tiles(const T *__
     for (long long t = blockIdx.x; t < bp.ntiles; t += gridDim.x) tile2_update<TW, TH, T>(in, out, bp, t, G);
 }
 
+// D2Q9, shape 0: one item of the table by one warp (rows2.cuh). In the persistent form
+// the state is read past L1 (other CTAs wrote it during the launch).
+template <int NS, typename T, bool COHERENT>
+__device__ __forceinline__ void rows2_update(const T *in, T *out, const BatchRows &it, long long fstride, bool wait) {
+    const rows2::Dom2 dm{it.nx, it.ny, it.off, fstride, it.s, it.a};
+    const rows2::Walls2 wl{};
+    const rows2::Force2 fc{};
+    const rows2::March<NS, T, COHERENT, false, false, false, false> m(in, out, dm, it.x0, wl, fc, 0.f, 0.f);
+    if (wait) asm volatile("griddepcontrol.wait;" ::: "memory");
+    m.rows(it.ya, it.yb);
+}
+// One warp per CTA with two strips a warp (its row arithmetic is then uniform), four with one
+// (fewer CTAs to start).
+constexpr int rows_warps(int ns) { return ns == 1 ? 4 : 1; }
+template <int NS, typename T>
+__global__ void __launch_bounds__(32 * rows_warps(NS)) k_batch_rows(const T *__restrict__ in, T *__restrict__ out,
+                                                                    BatchParams bp) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const long long t = rows_warps(NS) == 1 ? (long long)blockIdx.x
+                                            : (long long)blockIdx.x * rows_warps(NS) + (threadIdx.x >> 5);
+    if (t < bp.ntiles) rows2_update<NS, T, false>(in, out, bp.rows2[t], bp.fstride, true);
+}
+
 template <int Q, typename T>
 __global__ void __launch_bounds__(kTile) k_batch_step(const T *__restrict__ in, T *__restrict__ out,
                                                       BatchParams bp) {
@@ -343,6 +374,22 @@ __global__ void __launch_bounds__(kTile) k_batch_persistent(T *buf0, T *buf1, Ba
         for (long long t = blockIdx.x; t < bp.ntiles; t += gridDim.x) tile_update<Q, T>(in, out, bp, t);
         if (s + 1 < nsteps) {
             // test hook: CTA 0 leaves without arriving, so the others' waits run out
+            if (bp.withhold_step == s && blockIdx.x == 0) return;
+            if (!grid_barrier(bp, (unsigned)(s + 1))) return;
+        }
+    }
+}
+
+template <int NS, typename T>
+__global__ void __launch_bounds__(kTile) k_batch_rows_persistent(T *buf0, T *buf1, BatchParams bp, long long nsteps,
+                                                                 int parity) {
+    for (long long s = 0; s < nsteps; ++s) {
+        const int cur = (int)((parity + s) & 1);
+        const T *in = cur ? buf1 : buf0;
+        T *out = cur ? buf0 : buf1;
+        for (long long t = blockIdx.x * (kTile / 32) + (threadIdx.x >> 5); t < bp.ntiles; t += gridDim.x * (kTile / 32))
+            rows2_update<NS, T, true>(in, out, bp.rows2[t], bp.fstride, false);
+        if (s + 1 < nsteps) {
             if (bp.withhold_step == s && blockIdx.x == 0) return;
             if (!grid_barrier(bp, (unsigned)(s + 1))) return;
         }
@@ -473,6 +520,50 @@ cudaError_t single_dispatch(int shape, const void *in, void *out, const StepPara
     return cudaErrorInvalidValue;
 }
 
+// D2Q9, shape 0
+template <int NS, typename T>
+cudaError_t rows_t(const void *in, void *out, void *b0, void *b1, const BatchParams &bp, long long nsteps, int parity,
+                   bool persistent, cudaStream_t st) {
+    if (!persistent) {
+        const int w = rows_warps(NS);
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)((bp.ntiles + w - 1) / w));
+        cfg.blockDim = dim3(32 * w);
+        cfg.stream = st;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        return cudaLaunchKernelEx(&cfg, k_batch_rows<NS, T>, (const T *)in, (T *)out, bp);
+    }
+    static DevSlots cap;
+    const int g = max_grid(k_batch_rows_persistent<NS, T>, kTile, cap);
+    if (g < 1) return cudaErrorNotSupported;
+    const long long need = (bp.ntiles + kTile / 32 - 1) / (kTile / 32);
+    const long long grid = need < g ? need : g;
+    T *p0 = (T *)b0, *p1 = (T *)b1;
+    BatchParams q = bp;
+    void *args[] = {&p0, &p1, &q, &nsteps, &parity};
+    return cudaLaunchCooperativeKernel((const void *)k_batch_rows_persistent<NS, T>, dim3((unsigned)grid), dim3(kTile),
+                                       args, 0, st);
+}
+cudaError_t rows_storage(int storage, const void *in, void *out, void *b0, void *b1, const BatchParams &bp,
+                         long long nsteps, int parity, bool persistent, cudaStream_t st) {
+    switch (storage) {
+        case STORE_F32:
+            return bp.ns == 1 ? rows_t<1, float>(in, out, b0, b1, bp, nsteps, parity, persistent, st)
+                              : rows_t<2, float>(in, out, b0, b1, bp, nsteps, parity, persistent, st);
+        case STORE_BF16:
+            return bp.ns == 1 ? rows_t<1, __nv_bfloat16>(in, out, b0, b1, bp, nsteps, parity, persistent, st)
+                              : rows_t<2, __nv_bfloat16>(in, out, b0, b1, bp, nsteps, parity, persistent, st);
+        case STORE_F16:
+            return bp.ns == 1 ? rows_t<1, __half>(in, out, b0, b1, bp, nsteps, parity, persistent, st)
+                              : rows_t<2, __half>(in, out, b0, b1, bp, nsteps, parity, persistent, st);
+    }
+    return cudaErrorInvalidValue;
+}
+
 template <int Q, typename T>
 cudaError_t persistent_t(void *b0, void *b1, const BatchParams &bp, long long nsteps, int parity,
                          cudaStream_t st) {
@@ -488,19 +579,30 @@ cudaError_t persistent_t(void *b0, void *b1, const BatchParams &bp, long long ns
 }
 
 template <typename T>
-cudaError_t step_t(int Q, const void *in, void *out, const BatchParams &bp, cudaStream_t st) {
+cudaError_t step_t(const void *in, void *out, const BatchParams &bp, cudaStream_t st) {
     const long long cap = (long long)device_sms() * 8;
     const unsigned grid = (unsigned)(bp.ntiles < cap ? bp.ntiles : cap);
-    if (Q == 9)
-        k_batch_step<9, T><<<grid, kTile, 0, st>>>((const T *)in, (T *)out, bp);
-    else
-        k_batch_step<19, T><<<grid, kTile, 0, st>>>((const T *)in, (T *)out, bp);
+    k_batch_step<19, T><<<grid, kTile, 0, st>>>((const T *)in, (T *)out, bp);
     return cudaGetLastError();
 }
 
 }  // namespace
 
 int batch_tile() { return kTile; }
+int batch_rows_strip() { return rows2::kHalf; }
+// the cut of one domain (rows2.cuh) over the whole ensemble's strips, for the warps the GPU
+// holds (28 a SM of the one-strip form, 23 of the other). 256 domains of 32 to 512 nodes a
+// side: 17 rows 37.7 us a step, 4 rows 46.3, 64 rows 45.2, one strip a warp 42.4 at best.
+void batch_rows_cut(const BatchDomain *doms, int n, int *ns, int *rows) {
+    long long w1 = 0, w2 = 0;
+    for (int b = 0; b < n; ++b) {
+        w1 += (long long)((doms[b].nx - 1) / rows2::kHalf + 1) * doms[b].ny;
+        w2 += (long long)((doms[b].nx - 1) / (2 * rows2::kHalf) + 1) * doms[b].ny;
+    }
+    const rows2::Cut c = rows2::cut_rows(w1, w2, 28LL * 152, 23LL * 152);
+    *ns = c.ns;
+    *rows = c.rows;
+}
 int batch_shapes() { return kNumShapes; }
 void batch_shape(int k, int *tw, int *th) {
     const int i = k >= 0 && k < kNumShapes ? k : 0;
@@ -537,10 +639,11 @@ cudaError_t launch_batch_step(int Q, int storage, const void *in, void *out, con
         if (!batch_shape_supported(Q, storage, bp.shape)) return cudaErrorInvalidValue;
         return tiles_storage(storage, in, out, nullptr, nullptr, bp, 1, 0, false, st);
     }
+    if (Q == 9) return rows_storage(storage, in, out, nullptr, nullptr, bp, 1, 0, false, st);
     switch (storage) {
-        case STORE_F32: return step_t<float>(Q, in, out, bp, st);
-        case STORE_BF16: return step_t<__nv_bfloat16>(Q, in, out, bp, st);
-        case STORE_F16: return step_t<__half>(Q, in, out, bp, st);
+        case STORE_F32: return step_t<float>(in, out, bp, st);
+        case STORE_BF16: return step_t<__nv_bfloat16>(in, out, bp, st);
+        case STORE_F16: return step_t<__half>(in, out, bp, st);
     }
     return cudaErrorInvalidValue;
 }
@@ -553,18 +656,11 @@ cudaError_t launch_batch_persistent(int Q, int storage, void *buf0, void *buf1, 
         if (!batch_shape_supported(Q, storage, bp.shape)) return cudaErrorInvalidValue;
         return tiles_storage(storage, nullptr, nullptr, buf0, buf1, bp, nsteps, parity, true, st);
     }
-    if (Q == 9) {
-        switch (storage) {
-            case STORE_F32: return persistent_t<9, float>(buf0, buf1, bp, nsteps, parity, st);
-            case STORE_BF16: return persistent_t<9, __nv_bfloat16>(buf0, buf1, bp, nsteps, parity, st);
-            case STORE_F16: return persistent_t<9, __half>(buf0, buf1, bp, nsteps, parity, st);
-        }
-    } else {
-        switch (storage) {
-            case STORE_F32: return persistent_t<19, float>(buf0, buf1, bp, nsteps, parity, st);
-            case STORE_BF16: return persistent_t<19, __nv_bfloat16>(buf0, buf1, bp, nsteps, parity, st);
-            case STORE_F16: return persistent_t<19, __half>(buf0, buf1, bp, nsteps, parity, st);
-        }
+    if (Q == 9) return rows_storage(storage, nullptr, nullptr, buf0, buf1, bp, nsteps, parity, true, st);
+    switch (storage) {
+        case STORE_F32: return persistent_t<19, float>(buf0, buf1, bp, nsteps, parity, st);
+        case STORE_BF16: return persistent_t<19, __nv_bfloat16>(buf0, buf1, bp, nsteps, parity, st);
+        case STORE_F16: return persistent_t<19, __half>(buf0, buf1, bp, nsteps, parity, st);
     }
     return cudaErrorInvalidValue;
 }

@@ -56,11 +56,25 @@ struct BatchTile {
 struct BatchTile2 {
     int dom, x0, y0, pad;
 };
+// D2Q9, shape 0: the item of a warp that marches along y (rows2.cuh): the strips of a
+// domain from column x0, rows [ya, yb); what it needs of the domain stands in it
+struct BatchRows {
+    long long off;  // the domain's first node (packed index)
+    int nx, ny;
+    int x0, ya, yb;
+    float s, a;
+    int pad[3];
+};
+// strips per warp (1 or 2) and rows per item for an ensemble
+void batch_rows_cut(const BatchDomain *doms, int n, int *ns, int *rows);
+int batch_rows_strip();  // columns of a strip
 struct BatchParams {
     const BatchDomain *doms;
     const BatchTile *tiles;
     const BatchTile2 *tiles2;  // same storage as tiles, used when shape > 0
-    int shape;                 // 0: 1D tiles of batch_tile() nodes; k > 0: 2D shape k
+    const BatchRows *rows2;    // same storage, used for D2Q9 and shape 0
+    int ns;                    // strips per warp of rows2
+    int shape;                 // 0: rows2 (D2Q9) or 1D tiles of batch_tile() nodes; k > 0: 2D shape k
     long long ntiles;
     long long fstride;
     unsigned *bar_count;  // followed by the barrier generation word

@@ -72,10 +72,12 @@ struct lwacm_ctx {
     // batched domains (nbatch > 0): packed one after the other
     int nbatch = 0;
     std::vector<BatchDomain> doms;
-    std::vector<BatchTile> tiles;    // 1D tiles (shape 0)
+    std::vector<BatchTile> tiles;    // 1D tiles (D3Q19, shape 0)
+    std::vector<BatchRows> rows2;    // strips and runs of rows (D2Q9, shape 0)
+    int rows_ns = 1;                 // strips per warp of rows2
     std::vector<BatchTile2> tiles2;  // 2D tiles of the current shape (shape > 0)
     int batch_shape = 0;
-    size_t tiles_cap = 0;  // table entries reserved in the workspace (largest over the shapes)
+    size_t tiles_cap = 0;  // table bytes reserved in the workspace (largest over the shapes)
     size_t off_doms = 0, off_tiles = 0, off_bar = 0;
     int batch_mode = 0;  // 0: one launch per step (graphs), 1: one persistent launch
     long long withhold = -1;
@@ -131,7 +133,7 @@ void layout(lwacm_ctx *c) {
         c->off_doms = off;
         off = align_up(off + sizeof(BatchDomain) * c->doms.size(), kAlign);
         c->off_tiles = off;
-        off = align_up(off + 16 * c->tiles_cap, kAlign);
+        off = align_up(off + c->tiles_cap, kAlign);
         c->off_bar = off;
         off = align_up(off + 16, kAlign);
     }
@@ -251,11 +253,37 @@ void build_tiles2(const lwacm_ctx *c, int k, std::vector<BatchTile2> &out) {
             for (int x = 0; x < c->doms[b].nx; x += tw) out.push_back(BatchTile2{b, x, y, 0});
 }
 
+// strips and runs of rows over every domain (D2Q9, shape 0)
+void build_rows2(lwacm_ctx *c) {
+    int rows = 1;
+    batch_rows_cut(c->doms.data(), c->nbatch, &c->rows_ns, &rows);
+    const int width = c->rows_ns * batch_rows_strip();
+    c->rows2.clear();
+    for (const BatchDomain &d : c->doms)
+        for (int y = 0; y < d.ny; y += rows)
+            for (int x = 0; x < d.nx; x += width) {
+                BatchRows r = {};
+                r.off = d.off;
+                r.nx = d.nx;
+                r.ny = d.ny;
+                r.x0 = x;
+                r.ya = y;
+                r.yb = d.ny - y > rows ? y + rows : d.ny;
+                r.s = d.s;
+                r.a = d.a;
+                c->rows2.push_back(r);
+            }
+}
+
 // upload the tile table of the current shape (host tables are pageable: synchronise)
 lwacm_status upload_tiles(lwacm_ctx *c) {
     if (c->batch_shape > 0) {
         build_tiles2(c, c->batch_shape, c->tiles2);
         CK(c, cudaMemcpyAsync(c->ws + c->off_tiles, c->tiles2.data(), sizeof(BatchTile2) * c->tiles2.size(),
+                              cudaMemcpyHostToDevice, c->stream),
+           "tile table");
+    } else if (c->Q == 9) {
+        CK(c, cudaMemcpyAsync(c->ws + c->off_tiles, c->rows2.data(), sizeof(BatchRows) * c->rows2.size(),
                               cudaMemcpyHostToDevice, c->stream),
            "tile table");
     } else {
@@ -272,8 +300,10 @@ BatchParams batch_params(lwacm_ctx *c) {
     bp.doms = (const BatchDomain *)(c->ws + c->off_doms);
     bp.tiles = (const BatchTile *)(c->ws + c->off_tiles);
     bp.tiles2 = (const BatchTile2 *)(c->ws + c->off_tiles);
+    bp.rows2 = (const BatchRows *)(c->ws + c->off_tiles);
+    bp.ns = c->rows_ns;
     bp.shape = c->batch_shape;
-    bp.ntiles = (long long)(c->batch_shape > 0 ? c->tiles2.size() : c->tiles.size());
+    bp.ntiles = (long long)(c->batch_shape > 0 ? c->tiles2.size() : (c->Q == 9 ? c->rows2.size() : c->tiles.size()));
     bp.fstride = c->Nal;
     bp.bar_count = (unsigned *)(c->ws + c->off_bar);
     bp.bar_gen = bp.bar_count + 1;
@@ -532,7 +562,7 @@ lwacm_status lwacm_batch_create(int lattice, int n, const int *nx, const int *ny
             d.n = (long long)nx[b] * ny[b] * z;
             d.s = (float)(18.0 * nu[b]);  // Eq. ACM2.0nu: s = 18 nu, a = 1 - 6 nu
             d.a = (float)(1.0 - 6.0 * nu[b]);
-            for (long long t = 0; t < d.n; t += tile) {
+            for (long long t = 0; lattice == LWACM_D3Q19 && t < d.n; t += tile) {
                 BatchTile bt;
                 bt.dom = b;
                 bt.pad = 0;
@@ -546,12 +576,14 @@ lwacm_status lwacm_batch_create(int lattice, int n, const int *nx, const int *ny
         return LWACM_E_NOMEM;
     }
     try {
-        c->tiles_cap = c->tiles.size();
+        c->tiles_cap = sizeof(BatchTile) * c->tiles.size();
         if (lattice == LWACM_D2Q9) {
+            build_rows2(c);
+            c->tiles_cap = sizeof(BatchRows) * c->rows2.size();
             std::vector<BatchTile2> t2;
             for (int k = 1; k < batch_shapes(); ++k) {
                 build_tiles2(c, k, t2);
-                c->tiles_cap = std::max(c->tiles_cap, t2.size());
+                c->tiles_cap = std::max(c->tiles_cap, sizeof(BatchTile2) * t2.size());
             }
         }
     } catch (...) {

@@ -54,8 +54,8 @@ inline int cta_warps(int nx) {
 struct Cut {
     int ns, rows;
 };
-inline Cut cut_domain(int nx, int ny, long long room1, long long room2) {
-    const long long w1 = (long long)((nx - 1) / kHalf + 1) * ny, w2 = (long long)((nx - 1) / (2 * kHalf) + 1) * ny;
+// w1, w2: strips (of one, of two) times rows in all
+inline Cut cut_rows(long long w1, long long w2, long long room1, long long room2) {
     const long long once1 = (w1 - 1) / room1 + 1, once2 = (w2 - 1) / room2 + 1;
     Cut c{1, (int)once1};
     if (once1 > 5) {
@@ -71,6 +71,10 @@ inline Cut cut_domain(int nx, int ny, long long room1, long long room2) {
                 if (cost < best) best = cost, c.rows = h;
             }
     }
+    return c;
+}
+inline Cut cut_domain(int nx, int ny, long long room1, long long room2) {
+    Cut c = cut_rows((long long)((nx - 1) / kHalf + 1) * ny, (long long)((nx - 1) / (2 * kHalf) + 1) * ny, room1, room2);
     if (c.rows > ny) c.rows = ny;
     return c;
 }

@@ -25,7 +25,7 @@ OPT_RHO0, OPT_STORAGE, OPT_GRAPH_CHUNK, OPT_KERNEL = 6, 7, 8, 9
 OPT_BATCH_MODE, OPT_TEST_WITHHOLD, OPT_FORCE_FIELD, OPT_BATCH_TILE, OPT_NU_P = 10, 11, 12, 13, 14
 OPT_SCALAR_ALPHA, OPT_BULK_GAMMA, OPT_SEMI_IMPLICIT = 15, 16, 17
 OPT_STOCHASTIC_ROUNDING = 18
-# 2D tile shapes of the D2Q9 batched kernel (LWACM_OPT_BATCH_TILE 1..6); 0 = 1D runs
+# 2D tile shapes of the D2Q9 batched kernel (LWACM_OPT_BATCH_TILE 1..6); 0 = strips (1D runs in 3D)
 BATCH_TILE_SHAPES = {0: None, 1: (30, 6), 2: (30, 14), 3: (62, 6), 4: (30, 30), 5: (62, 14), 6: (126, 6)}
 
 STATUS_NAMES = {OK: "OK", E_ARG: "E_ARG", E_RANGE: "E_RANGE", E_STATE: "E_STATE",
@@ -420,7 +420,8 @@ class LwacmBatch(Lwacm):
     Fields are packed domain after domain; set_domains / get_domains pack and
     unpack per-domain numpy arrays. mode 0: one launch per step (graphs); mode 1:
     one persistent cooperative launch per step() call. tile: LWACM_OPT_BATCH_TILE
-    (0 = runs of 256 nodes; 1..6 = the 2D shapes of BATCH_TILE_SHAPES, D2Q9).
+    (0 = strips marched along y for D2Q9, runs of 256 nodes for D3Q19; 1..6 = the 2D
+    shapes of BATCH_TILE_SHAPES, D2Q9).
     """
 
     def __init__(self, lattice, dims, nus, *, storage=F32, mode=0, tile=0, graph_chunk=None,

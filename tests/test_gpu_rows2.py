@@ -99,3 +99,28 @@ def test_rows_kernel_carries_extreme_values(lw, field, bad):
         assert np.array_equal(np.isnan(x), np.isnan(y)) and np.array_equal(np.isinf(x), np.isinf(y))
         ok = np.isfinite(y) & (np.abs(y) < 1e3)
         assert np.allclose(x[ok], y[ok], rtol=0, atol=1e-3)
+
+
+@pytest.mark.parametrize("storage", [0, 1, 2])
+@pytest.mark.parametrize("scale", [1, 12])
+def test_ensemble_strips_equal_single_domains(lw, storage, scale):
+    """An ensemble's strips give each domain the fields it has alone, bit for bit, in both
+    launch forms: a node's sums do not depend on how its domain is cut (scale 12: two strips
+    a warp)."""
+    dims = [(1, 1), (29, 3), (31, 7), (60, 5), (61, 2), (120, 40), (3, 90), (97, 61)]
+    dims = [(w * (scale if w > 60 else 1), h * (scale if w > 60 else 1)) for w, h in dims]
+    nus = [0.01 + 0.01 * b for b in range(len(dims))]
+    fields = [inputs.smooth_random((h, w), seed=30 + b, u_amp=0.04, d_amp=0.01) for b, (w, h) in enumerate(dims)]
+    for mode in (0, 1):
+        sim = lw.LwacmBatch(9, dims, nus, mode=mode, storage=storage)
+        sim.set_domains(fields)
+        sim.step(7)
+        got = sim.get_domains()
+        sim.close()
+        for (w, h), nu, f, g in zip(dims, nus, fields, got):
+            one = lw.Lwacm(9, w, h, 1, nu, storage=storage)
+            one.set_fields(*f)
+            one.step(7)
+            for x, y in zip(g, one.get_fields()):
+                assert np.array_equal(x, y), (mode, w, h)
+            one.close()
