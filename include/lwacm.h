@@ -88,7 +88,9 @@ enum {
     LWACM_OPT_GRAPH_CHUNK = 8, /* steps per captured CUDA graph in lwacm_step (even;
                                   0 disables graphs; default 64) */
     LWACM_OPT_KERNEL = 9,  /* interior kernel: 0 = automatic choice (default),
-                              1 = generic gather kernel, 5 = D3Q19 half-row TMA kernel
+                              1 = general kernel (any size and option; the plain
+                              D3Q19 scheme by warps that march along z, else a gather),
+                              5 = D3Q19 half-row TMA kernel
                               (needs the plain scheme, with or without a constant
                               acceleration but not a force field, nx = 128, 256 or
                               nx >= 72 a multiple of 4 (8 for BF16 / FP16 storage)
@@ -102,7 +104,8 @@ enum {
                               domains; not the scalar; tile shape from
                               LWACM_OPT_BATCH_TILE; 0: strips of columns marched along
                               y by warps). The automatic choice
-                              takes 5, else 6, else 1. */
+                              takes 5 (for the plain scheme on rows other than 128
+                              nodes the marching warps), else 6, else 1. */
     LWACM_OPT_BATCH_MODE = 10, /* batched contexts: 0 = one launch per step, replayed
                                   from CUDA graphs (default); 1 = one persistent
                                   cooperative launch per lwacm_step call, with a

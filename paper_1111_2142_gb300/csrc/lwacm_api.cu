@@ -41,6 +41,7 @@ struct lwacm_ctx {
     bool bulk = false;        // the variant is on: Tr+ - Tr^(e) is the field after the flow fields
     bool semi = false;        // semi-implicit pressure update (Eq. FDcompact_si)
     bool sr = false;          // BF16 / FP16 stores rounded stochastically (half-row kernel)
+    bool march = false;       // kernel 5, automatic choice: by warps that march along z (kernels_rows3.cu)
     bool scalar_rows = false; // the passive scalar on its own row-tiled kernel after the flow kernel
     int nsc = 0;              // fields stored after the flow fields: the scalar or the trace (0 or 1)
     long long N = 0, Nal = 0;
@@ -231,9 +232,16 @@ bool choose_kernel(lwacm_ctx *c) {
     static const char *sname[7] = {"tiles2d_d2q9_30x14", "tiles2d_d2q9_30x6",  "tiles2d_d2q9_30x14", "tiles2d_d2q9_62x6",
                                    "tiles2d_d2q9_30x30", "tiles2d_d2q9_62x14", "tiles2d_d2q9_126x6"};
     if (c->kernel != 5) c->scalar_rows = false;
+    // rows the half-row kernel takes, plain scheme: marching warps, which need no halves or
+    // segments (us a step, half-row / march: 256^3 137 / 129, 256 x 128 x 128 39 / 35, 384 x 256 x
+    // 256 278 / 178, 200 x 256 x 256 190 / 100), but for whole rows of one warp (128 x 256 x 256 65 /
+    // 77) and for a cavity whose x walls the half-row kernel applies
+    c->march = c->kernel == 5 && c->kernel_opt == 0 && !c->sr && !c->scalar_rows && rows3d_supported(p) && c->nx != 128 &&
+               (c->bc == LWACM_BC_PERIODIC || !half_xwalls(p));
     static const char *hname[2][2] = {{"half_d3q19_tma", "half_d3q19_tma+scalar_rows"},
                                       {"half_d3q19_tma+nu_p_sum", "half_d3q19_tma+nu_p_sum+scalar_rows"}};
-    c->kname = c->kernel == 5   ? hname[p.sdelta != 0.f ? 1 : 0][c->scalar_rows ? 1 : 0]
+    c->kname = c->march         ? "half_d3q19_march"
+               : c->kernel == 5 ? hname[p.sdelta != 0.f ? 1 : 0][c->scalar_rows ? 1 : 0]
                : c->kernel == 6 ? (dev && c->batch_shape == 0 ? "tiles2d_d2q9_rows" : sname[c->batch_shape < 7 ? c->batch_shape : 0])
                                 : gname[c->Q == 19 ? 1 : 0];
     return ok;
@@ -321,7 +329,8 @@ cudaError_t step_between(lwacm_ctx *c, const void *in, void *out, cudaStream_t s
     cudaError_t e = cudaSuccess;
     if (c->kernel == 5 && p.sdelta != 0.f) e = launch_nup_sum(c->storage, in, p.nup_p, p, st);
     if (e != cudaSuccess) return e;
-    e = c->kernel == 5               ? launch_step_half(c->Q, c->storage, in, out, pf, st)
+    e = c->march                     ? launch_step_rows3d(c->storage, in, out, p, st)
+                    : c->kernel == 5 ? launch_step_half(c->Q, c->storage, in, out, pf, st)
                     : c->kernel == 6 && c->batch_shape == 0 ? launch_step_rows2d(c->storage, in, out, p, st)
                     : c->kernel == 6 ? launch_step_tiles2d(c->Q, c->storage, c->batch_shape, in, out, p, st)
                                      : launch_step_generic(c->Q, c->storage, in, out, p, st);
@@ -330,7 +339,7 @@ cudaError_t step_between(lwacm_ctx *c, const void *in, void *out, cudaStream_t s
     // walls of a cavity whose lid is not on an x face
     if (c->bc != LWACM_BC_PERIODIC && c->kernel != 6) {
         StepParams pw = p;
-        pw.xfaces_done = c->kernel == 5 && half_xwalls(p) ? 1 : 0;
+        pw.xfaces_done = c->kernel == 5 && !c->march && half_xwalls(p) ? 1 : 0;
         e = launch_wall_pass(c->Q, c->storage, in, out, pw, st);
     }
     if (e == cudaSuccess && p.sr_ctr && c->kernel == 5) e = launch_sr_tick(p.sr_ctr, st);

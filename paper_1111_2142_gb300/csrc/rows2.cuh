@@ -123,6 +123,16 @@ __device__ __forceinline__ float from_right(float v) { return __shfl_down_sync(t
 __device__ __forceinline__ F2 from_left(F2 v) { return make_float2(from_left(v.x), from_left(v.y)); }
 __device__ __forceinline__ F2 from_right(F2 v) { return make_float2(from_right(v.x), from_right(v.y)); }
 
+// an element some bytes from a pointer that is uniform over the warp: a 32-bit offset of the
+// lane's own costs no address arithmetic
+template <typename T>
+__device__ __forceinline__ T *byte_at(T *p, unsigned bytes) {
+    return (T *)((char *)p + bytes);
+}
+template <typename T>
+__device__ __forceinline__ const T *byte_at(const T *p, unsigned bytes) {
+    return (const T *)((const char *)p + bytes);
+}
 // stored elements as loaded: widened when used, so that a load in flight holds nothing up
 template <bool COHERENT, typename T>
 __device__ __forceinline__ T ldraw(const T *p) {
