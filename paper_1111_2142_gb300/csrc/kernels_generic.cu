@@ -500,31 +500,202 @@ __global__ void k_from(const Ti *__restrict__ in, T *__restrict__ out, long long
 }
 
 // ---- FP64 diagnostics: per-block partials, then one block in fixed order ------
+//
+// GB300 has two FP64 lanes a SM and 128 FP32 ones, and the sums need 17 FP64 operations and
+// four conversions a node, so in FP64 they took 0.8 ms at 256^3 (40 us of memory). A thread
+// therefore keeps its sums as unevaluated sums of FP32 numbers, packed for two nodes, and turns
+// them into FP64 once at the end: every product is split exactly into its rounded value and the
+// rest (an FMA), every addition leaves its exact error (Knuth's TwoSum, D. E. Knuth, The Art of
+// Computer Programming 2, 4.2.2), which goes to the next component. Three components carry some
+// 70 bits, more than the FP64 sums did. The square of u + v (or u - v) is that of the exact sum.
+// Some 290 FP32 operations a node; the whole call at 256^3 192 us, before 789.
+// A thread whose values leave the range in which the splits are exact (an infinity, a NaN, an
+// overflow, velocities all below 2^-40) sums its nodes in FP64 instead, as diag_node does.
 constexpr int kDiagVals = 9;  // mass, jx, jy, jz, ke, max|u|^2, mpar, mperp, nonfinite
 
-template <typename T>
-__global__ void __launch_bounds__(256) k_diag_partial(const T *__restrict__ f, long long fstride,
-                                                      long long N, int has_z,
+__device__ __forceinline__ void diag_node(double (&acc)[kDiagVals], double d, double u, double v, double w, bool has_z) {
+    const double rho = 1.0 + d, uu = u * u + v * v + w * w;
+    acc[0] += d;
+    acc[1] += rho * u;
+    acc[2] += rho * v;
+    acc[3] += rho * w;
+    acc[4] += 0.5 * rho * uu;
+    acc[5] = fmax(acc[5], uu);
+    if (has_z) {
+        // Eq. 3Dmomenta, read for a lid moving along the x = y diagonal of the
+        // top z plane: components parallel / perpendicular to the lid (times sqrt 2)
+        acc[6] += 0.5 * (u + v) * (u + v);
+        acc[7] += 0.5 * (u - v) * (u - v);
+    }
+    if (!isfinite(d) || !isfinite(uu)) acc[8] += 1.0;
+}
+
+namespace sums {
+
+using F2 = float2;
+__device__ __forceinline__ F2 add(F2 a, F2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ F2 sub(F2 a, F2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
+__device__ __forceinline__ F2 mul(F2 a, F2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ F2 fma(F2 a, F2 b, F2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ F2 neg(F2 a) { return make_float2(-a.x, -a.y); }
+// a + b = s + the returned error, exactly
+__device__ __forceinline__ F2 two_sum(F2 a, F2 b, F2 &s) {
+    s = add(a, b);
+    const F2 t = sub(s, a);
+    return add(sub(a, sub(s, t)), sub(b, t));
+}
+__device__ __forceinline__ float two_sum(float a, float b, float &s) {
+    s = __fadd_rn(a, b);
+    const float t = __fsub_rn(s, a);
+    return __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
+}
+// a b = h + the returned error, exactly
+__device__ __forceinline__ F2 two_prod(F2 a, F2 b, F2 &h) {
+    h = mul(a, b);
+    return fma(a, b, neg(h));
+}
+struct Three {
+    F2 a{0.f, 0.f}, b{0.f, 0.f}, c{0.f, 0.f};
+    __device__ __forceinline__ void down(F2 e) { c = add(c, two_sum(b, e, b)); }
+    __device__ __forceinline__ void add1(F2 x) { down(two_sum(a, x, a)); }
+    __device__ __forceinline__ void add2(F2 h, F2 l) {
+        add1(h);
+        down(l);
+    }
+    // the pair's two sums as one, then in FP64
+    __device__ __forceinline__ double value() const {
+        float s, t;
+        const float e = two_sum(a.x, a.y, s), g = two_sum(b.x, b.y, t), h = two_sum(t, e, t);
+        return (double)s + ((double)t + (double)((c.x + c.y) + (g + h)));
+    }
+    __device__ __forceinline__ bool ok() const { return isfinite(a.x + a.y + b.x + b.y + c.x + c.y); }
+};
+// the sums of the nodes a thread takes, two at a time
+template <bool HAS_Z>
+struct Node2 {
+    Three mass, jx, jy, jz, ke, par, perp;  // ke: of rho |u|^2
+    double top = 0.0;           // max |u|^2
+    float near = 1e-45f, big = 0.f;  // the least |u|^2 worth forming in FP64; max |u|
+
+    __device__ __forceinline__ void momentum(Three &j, F2 d, F2 u) {  // u + d u
+        j.add1(u);
+        F2 h;
+        const F2 e = two_prod(d, u, h);
+        j.add2(h, e);
+    }
+    __device__ __forceinline__ void square(Three &t, F2 u, F2 v) {  // (u + v)^2
+        F2 s, h, g;
+        const F2 e = two_sum(u, v, s), l = two_prod(s, s, h), m = two_prod(add(s, s), e, g);
+        t.add2(h, l);
+        t.down(g);
+        t.c = add(t.c, fma(e, e, m));
+    }
+    __device__ __forceinline__ void top_of(float p, float u, float v, float w) {
+        big = fmaxf(big, fmaxf(fabsf(u), fmaxf(fabsf(v), fabsf(w))));
+        if (p >= near) {  // within the rounding of p of the greatest so far, or above
+            const double x = (double)u * u + (double)v * v + (double)w * w;
+            if (x > top) {
+                top = x;
+                near = p * (1.f - 4e-7f);
+            }
+        }
+    }
+    __device__ __forceinline__ void take(F2 d, F2 u, F2 v, F2 w) {
+        mass.add1(d);
+        momentum(jx, d, u);
+        momentum(jy, d, v);
+        if (HAS_Z) momentum(jz, d, w);
+        // |u|^2 = p + l, the parts of l added one by one (the last bits of squares are no random
+        // ones: their sum rounded for each node is off by 4 parts in 10^16 on average)
+        F2 p, q, h;
+        F2 l = two_prod(u, u, p);
+        ke.down(l);
+        F2 r = two_prod(v, v, h);
+        ke.down(r);
+        l = add(l, r);
+        r = two_sum(p, h, p);
+        ke.down(r);
+        l = add(l, r);
+        if (HAS_Z) {
+            r = two_prod(w, w, h);
+            ke.down(r);
+            l = add(l, r);
+            r = two_sum(p, h, p);
+            ke.down(r);
+            l = add(l, r);
+        }
+        ke.add1(p);
+        const F2 e = two_prod(d, p, q);
+        ke.add2(q, fma(d, l, e));
+        if (HAS_Z) {
+            square(par, u, v);
+            square(perp, u, neg(v));
+        }
+        top_of(p.x, u.x, v.x, w.x);
+        top_of(p.y, u.y, v.y, w.y);
+    }
+    __device__ __forceinline__ bool ok() const {
+        bool k = mass.ok() && jx.ok() && jy.ok() && ke.ok();
+        if (HAS_Z) k = k && jz.ok() && par.ok() && perp.ok();
+        return k && (big >= 9.1e-13f || big == 0.f);  // 2^-40
+    }
+    __device__ __forceinline__ void values(double (&acc)[kDiagVals]) const {
+        acc[0] = mass.value();
+        acc[1] = jx.value();
+        acc[2] = jy.value();
+        acc[3] = HAS_Z ? jz.value() : 0.0;
+        acc[4] = 0.5 * ke.value();
+        acc[5] = top;
+        acc[6] = HAS_Z ? 0.5 * par.value() : 0.0;
+        acc[7] = HAS_Z ? 0.5 * perp.value() : 0.0;
+    }
+};
+
+}  // namespace sums
+
+// F64: every node in FP64, for few nodes
+template <typename T, bool HAS_Z, bool F64>
+__global__ void __launch_bounds__(256, 2) k_diag_partial(const T *__restrict__ f, long long fstride, long long N,
                                                       double *__restrict__ partial) {
     double acc[kDiagVals] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < N;
-         i += (long long)gridDim.x * blockDim.x) {
-        const double d = ldf(f + i), u = ldf(f + fstride + i), v = ldf(f + 2 * fstride + i);
-        const double w = has_z ? (double)ldf(f + 3 * fstride + i) : 0.0;
-        const double rho = 1.0 + d, uu = u * u + v * v + w * w;
-        acc[0] += d;
-        acc[1] += rho * u;
-        acc[2] += rho * v;
-        acc[3] += rho * w;
-        acc[4] += 0.5 * rho * uu;
-        acc[5] = fmax(acc[5], uu);
-        if (has_z) {
-            // Eq. 3Dmomenta, read for a lid moving along the x = y diagonal of the
-            // top z plane: components parallel / perpendicular to the lid (times sqrt 2)
-            acc[6] += 0.5 * (u + v) * (u + v);
-            acc[7] += 0.5 * (u - v) * (u - v);
+    const long long t0 = (long long)blockIdx.x * blockDim.x + threadIdx.x, step = (long long)gridDim.x * blockDim.x;
+    const long long quads = F64 ? 0 : N / 4;  // fields start 256-byte aligned: four values a load
+    if (!F64) {
+        sums::Node2<HAS_Z> s;
+        const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
+        float4 d, u, v, w = z4;
+        if (t0 < quads) {
+            d = tile::ld4(f + 4 * t0);
+            u = tile::ld4(f + fstride + 4 * t0);
+            v = tile::ld4(f + 2 * fstride + 4 * t0);
+            if (HAS_Z) w = tile::ld4(f + 3 * fstride + 4 * t0);
         }
-        if (!isfinite(d) || !isfinite(uu)) acc[8] += 1.0;
+        for (long long i = t0; i < quads; i += step) {
+            float4 dn = z4, un = z4, vn = z4, wn = z4;  // the next four nodes, on their way meanwhile
+            if (i + step < quads) {
+                const long long k = 4 * (i + step);
+                dn = tile::ld4(f + k);
+                un = tile::ld4(f + fstride + k);
+                vn = tile::ld4(f + 2 * fstride + k);
+                if (HAS_Z) wn = tile::ld4(f + 3 * fstride + k);
+            }
+            s.take(make_float2(d.x, d.y), make_float2(u.x, u.y), make_float2(v.x, v.y), make_float2(w.x, w.y));
+            s.take(make_float2(d.z, d.w), make_float2(u.z, u.w), make_float2(v.z, v.w), make_float2(w.z, w.w));
+            d = dn, u = un, v = vn, w = wn;
+        }
+        if (t0 >= quads) {
+        } else if (s.ok()) {
+            s.values(acc);
+        } else {
+            for (long long i = t0; i < quads; i += step)
+                for (long long k = 4 * i; k < 4 * i + 4; ++k)
+                    diag_node(acc, ldf(f + k), ldf(f + fstride + k), ldf(f + 2 * fstride + k),
+                              HAS_Z ? ldf(f + 3 * fstride + k) : 0.f, HAS_Z);
+        }
+    }
+    for (long long k = 4 * quads + t0; k < N; k += step) {  // all of them, or the last three at most
+        diag_node(acc, ldf(f + k), ldf(f + fstride + k), ldf(f + 2 * fstride + k), HAS_Z ? ldf(f + 3 * fstride + k) : 0.f,
+                  HAS_Z);
     }
     __shared__ double sh[kDiagVals][256];
     for (int v = 0; v < kDiagVals; ++v) sh[v][threadIdx.x] = acc[v];
@@ -686,7 +857,15 @@ cudaError_t launch_convert_out(int storage, int dst_dtype, const void *src, void
 template <typename T>
 static cudaError_t diag_t(const void *f, long long fstride, long long N, int has_z, double *partial,
                           double *out, cudaStream_t st) {
-    k_diag_partial<T><<<kDiagBlocks, 256, 0, st>>>((const T *)f, fstride, N, has_z, partial);
+    // in FP64 throughout below 2^18 nodes, where the launches and the read-back are most of it
+    // and a thread's own sums take as long to turn into FP64 as its nodes (the call in us, FP64 /
+    // expansions: 48^3 41 / 43, 60^3 42 / 41, 72^3 53 / 44, 128^3 128 / 66, 256^3 789 / 192)
+    const bool f64 = N < (1 << 18);
+    const T *p = (const T *)f;
+    if (has_z && f64) k_diag_partial<T, true, true><<<kDiagBlocks, 256, 0, st>>>(p, fstride, N, partial);
+    if (has_z && !f64) k_diag_partial<T, true, false><<<kDiagBlocks, 256, 0, st>>>(p, fstride, N, partial);
+    if (!has_z && f64) k_diag_partial<T, false, true><<<kDiagBlocks, 256, 0, st>>>(p, fstride, N, partial);
+    if (!has_z && !f64) k_diag_partial<T, false, false><<<kDiagBlocks, 256, 0, st>>>(p, fstride, N, partial);
     k_diag_final<<<1, 256, 0, st>>>(partial, kDiagBlocks, out);
     return cudaGetLastError();
 }
