@@ -95,6 +95,10 @@ cudaError_t launch_step_tiles2d(int Q, int storage, int shape, const void *in, v
                                 cudaStream_t st);
 // the D2Q9 update by warps that march along y (kernels_rows2.cu), where tiles2d_supported()
 cudaError_t launch_step_rows2d(int storage, const void *in, void *out, const StepParams &p, cudaStream_t st);
+// several steps of a small D2Q9 domain in one launch (kernels_cluster2.cu), the same fields as
+// that many launch_step_rows2d
+bool cluster2d_supported(const StepParams &p);
+cudaError_t launch_cluster2d(int storage, const void *in, void *out, const StepParams &p, int steps, cudaStream_t st);
 // the plain D3Q19 scheme by warps that march along z (kernels_rows3.cu), any size
 bool rows3d_supported(const StepParams &p);
 cudaError_t launch_step_rows3d(int storage, const void *in, void *out, const StepParams &p, cudaStream_t st);

@@ -1,0 +1,72 @@
+"""Several steps of a small D2Q9 domain in one launch of a cluster (kernels_cluster2.cu): the
+same fields, bit for bit, as single steps on the marching kernel, which the oracle checks."""
+import numpy as np
+import pytest
+
+from paper_1111_2142_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+# fewer rows than CTAs, one column, one node to two nodes a thread, uneven rows, the largest
+SHAPES = [(1, 1), (7, 1), (1, 7), (2, 2), (3, 29), (16, 31), (17, 33), (33, 60), (128, 128), (150, 100), (16, 1664)]
+
+
+@pytest.fixture(scope="module")
+def lw():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("needs a GPU")
+    from paper_1111_2142_gb300 import lwacm
+    return lwacm
+
+
+def both(lw, shape, T, bc=0, nu_p=None, **kw):
+    ny, nx = shape
+    f = inputs.smooth_random(shape, seed=71, u_amp=0.05, d_amp=0.01)
+    out = []
+    for calls in ([T], [1] * T):
+        sim = lw.Lwacm(9, nx, ny, 1, 0.02, bc, lid=(0.05, 0.01) if bc else None, **kw)
+        if nu_p:
+            sim.set_option(lw.OPT_NU_P, nu_p)
+        sim.set_fields(*f)
+        for n in calls:
+            sim.step(n)
+        assert sim.step_count() == T
+        got = list(sim.get_fields())
+        if kw.get("bulk_gamma"):
+            got.append(sim.get_trace())
+        sim.close()
+        out.append(got)
+    for a, b in zip(*out):
+        assert np.array_equal(a, b), (shape, bc, nu_p, kw)
+
+
+@pytest.mark.parametrize("storage", [0, 1, 2])
+@pytest.mark.parametrize("shape", SHAPES)
+def test_cluster_equals_single_steps(lw, shape, storage):
+    both(lw, shape, 5, storage=storage)
+    both(lw, shape, 6, storage=storage, force=(1e-4, 2e-5))
+    both(lw, shape, 5, storage=storage, nu_p=0.1)
+    both(lw, shape, 5, storage=storage, bulk_gamma=0.4)
+    both(lw, shape, 6, storage=storage, bulk_gamma=0.3, nu_p=0.08)
+    if min(shape) >= 2:
+        both(lw, shape, 5, bc=1, storage=storage)
+        both(lw, shape, 5, bc=2, storage=storage, force=(1e-4, 0.0))
+
+
+def test_cluster_then_single_steps_and_long_runs(lw):
+    """Any split of a run gives the same fields: more steps than one launch takes, odd
+    remainders, a graph prepared for the whole run."""
+    f = inputs.smooth_random((20, 24), seed=72, u_amp=0.03, d_amp=0.005)
+    out = []
+    for calls in ([8192 + 131], [1, 64, 3, 8192 + 63]):
+        sim = lw.Lwacm(9, 24, 20, 1, 0.02)
+        sim.set_fields(*f)
+        sim.prepare(sum(calls))
+        for n in calls:
+            sim.step(n)
+        assert sim.step_count() == 8192 + 131
+        out.append(sim.get_fields())
+        sim.close()
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
