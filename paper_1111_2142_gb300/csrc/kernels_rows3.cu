@@ -1,5 +1,5 @@
 // D3Q19 update by warps that march along z, for domains of any size: the moment form of
-// Eq. ACM2.0 (lwacm_core.cuh) with forcing, every axis periodic.
+// Eq. ACM2.0 (lwacm_core.cuh) with walls and forcing.
 //
 // A warp takes an item: a strip of 30 columns, a tile of four rows and a run of planes.
 // Lane l holds column x0 + l - 1 (lanes 0 and 31 are the strip's neighbours) of the four
@@ -51,6 +51,10 @@ struct Dom3 {
     float g[3];       // constant acceleration (Eq. force)
     int forced;
     const float *field;  // per-node acceleration
+    // half-way walls (Eqs. ACM2.0cccbb2 / ACM2.0ccccbb) on both ends of x, y, z; the top of the lid
+    // axis (1 or 2) moves with the lid velocity; wall = 36 nu rho0
+    int wx, wy, wz, lid_axis;
+    float wall, lid[3];
 };
 
 enum { FIRST = 0, START = 1, MID = 2, LAST = 3 };
@@ -65,7 +69,7 @@ struct Sum3 {
     F2 D, X, Y, Z;
 };
 
-template <typename T, bool FIELD>
+template <typename T, bool FIELD, bool WALLS>
 struct March3 {
     const T *in;
     T *out;
@@ -74,6 +78,8 @@ struct March3 {
     float odd;
     unsigned off, lo, hi;  // bytes to row y0 at the lane's column in a plane; to the rows below and above the tile
     bool st;
+    // WALLS: the lane's column lies at an x wall; the tile's first / last row at a y wall
+    bool e0 = false, eN = false, low = false, top = false, edge = false;
 
     __device__ __forceinline__ March3(const T *in_, T *out_, const Dom3 &dm_, int x0, int y0)
         : in(in_), out(out_), dm(dm_), plane((long long)dm_.nx * dm_.ny), odd(dm_.s * (2.f / 9.f)) {
@@ -83,6 +89,22 @@ struct March3 {
         lo = ((unsigned)(y0 > 0 ? y0 - 1 : dm.ny - 1) * nx + xw) * (unsigned)sizeof(T);
         hi = ((unsigned)(y0 + kTile < dm.ny ? y0 + kTile : 0) * nx + xw) * (unsigned)sizeof(T);
         st = lane >= 1 && lane <= kStrip && x < dm.nx;
+        if (WALLS) {
+            e0 = dm.wx && x == 0;
+            eN = dm.wx && x == dm.nx - 1;
+            edge = dm.wx && (x0 == 0 || x0 + kStrip >= dm.nx);
+            low = dm.wy && y0 == 0;
+            top = dm.wy && y0 + kTile == dm.ny;
+        }
+    }
+    // from x - 1 / x + 1; nothing comes through a wall
+    __device__ __forceinline__ F2 left(F2 v) const {
+        const F2 t = from_left(v);
+        return WALLS && e0 ? bc<F2>(0.f) : t;
+    }
+    __device__ __forceinline__ F2 right(F2 v) const {
+        const F2 t = from_right(v);
+        return WALLS && eN ? bc<F2>(0.f) : t;
     }
 
     struct Raw {
@@ -141,7 +163,7 @@ struct March3 {
         if (OWN) {
             F2 xp, xm;
             pair(n, n.u, false, xp, xm);
-            const F2 l = from_left(xp), r = from_right(xm);
+            const F2 l = left(xp), r = right(xm);
             const F2 m = fma(dm.a, d, bc<F2>(dm.am1));  // a rho u = u + m u (post_combine)
             C.Z = add(fma(m, n.w, C.D), n.w);           // so far every link came with c_z = +1
             C.X = add(fma(m, n.u, add(C.X, sub(l, r))), n.u);
@@ -159,13 +181,13 @@ struct March3 {
             }
         }
         if (DOWN) {
-            const F2 l = from_left(pm), r = from_right(mm), s = add(zm, add(l, r));
+            const F2 l = left(pm), r = right(mm), s = add(zm, add(l, r));
             P.D = add(P.D, s);
             P.X = add(P.X, sub(l, r));
             P.Z = sub(P.Z, s);
         }
         if (UP) {
-            const F2 l = from_left(pp), r = from_right(mp);
+            const F2 l = left(pp), r = right(mp);
             N.D = add(zp, add(l, r));
             N.X = sub(l, r);
         }
@@ -178,10 +200,10 @@ struct March3 {
             pair(n, n.v, false, yp, ym);
             pair(n, add(n.u, n.v), true, pp, mm);  // (1,1,0) (-1,-1,0)
             pair(n, sub(n.u, n.v), true, pm, mp);  // (1,-1,0) (-1,1,0)
-            F2 l = from_left(pp), r = from_right(mp);
+            F2 l = left(pp), r = right(mp);
             up.s = add(yp, add(l, r));
             up.t = sub(l, r);
-            l = from_left(pm), r = from_right(mm);
+            l = left(pm), r = right(mm);
             dn.s = add(ym, add(l, r));
             dn.t = sub(l, r);
         }
@@ -194,12 +216,89 @@ struct March3 {
     template <int MODE>
     __device__ __forceinline__ void halo(const Node &n, Send &h) const {
         if (MODE == START || MODE == MID) {
-            const F2 l = from_left(plus(n, add(n.v, n.u), true)), r = from_right(plus(n, sub(n.v, n.u), true));
+            const F2 l = left(plus(n, add(n.v, n.u), true)), r = right(plus(n, sub(n.v, n.u), true));
             h.s = add(plus(n, n.v, false), add(l, r));
             h.t = sub(l, r);
         }
         if (MODE != LAST) h.p = plus(n, add(n.v, n.w), true);
         if (MODE == MID || MODE == LAST) h.m = plus(n, sub(n.v, n.w), true);
+        if (WALLS && low) h.s.x = h.t.x = h.p.x = h.m.x = 0.f;
+        if (WALLS && top) h.s.y = h.t.y = h.p.y = h.m.y = 0.f;
+    }
+    // WALLS: what the walls send back to plane z of the row pair k (tile rows k and k + 2): for each
+    // link whose source lies beyond a wall the node's own value of the opposite link, plus the lid
+    // term at the top of the lid axis; a link that leaves through two walls is taken at the z wall,
+    // else at the y wall
+    __device__ __forceinline__ void bounce(const Node &n, int k, int z, Sum3 &C) const {
+        const bool z0 = dm.wz && z == 0, zN = dm.wz && z == dm.nz - 1;
+        const bool y0 = low && k == 0, yN = top && k == 1;  // the pair's first / second row
+        if (!(z0 || zN || y0 || yN || edge)) return;
+        F2 zp, zm, xzp, xzm, zxp, zxm, yzp, yzm, zyp, zym;
+        pair(n, add(n.u, n.w), true, xzp, xzm);  // (1,0,1) (-1,0,-1)
+        pair(n, sub(n.u, n.w), true, zxp, zxm);  // (1,0,-1) (-1,0,1)
+        pair(n, add(n.v, n.w), true, yzp, yzm);  // (0,1,1) (0,-1,-1)
+        pair(n, sub(n.v, n.w), true, zyp, zym);  // (0,1,-1) (0,-1,1)
+        if (z0 || zN) pair(n, n.w, false, zp, zm);
+        if (z0) {
+            const F2 s = add(zm, add(add(xzm, zxp), add(yzm, zyp)));
+            C.D = add(C.D, s);
+            C.Z = add(C.Z, s);
+            C.X = add(C.X, sub(xzm, zxp));
+            C.Y = add(C.Y, sub(yzm, zyp));
+        }
+        if (zN) {
+            const float w = dm.lid_axis == 2 ? dm.wall * (1.f / 36.f) : 0.f;
+            const F2 a = add(zp, -2.f * w * dm.lid[2]);
+            const F2 b = add(zxm, w * (dm.lid[0] - dm.lid[2])), c = add(xzp, w * (-dm.lid[0] - dm.lid[2]));
+            const F2 d = add(zym, w * (dm.lid[1] - dm.lid[2])), e = add(yzp, w * (-dm.lid[1] - dm.lid[2]));
+            const F2 s = add(a, add(add(b, c), add(d, e)));
+            C.D = add(C.D, s);
+            C.Z = sub(C.Z, s);
+            C.X = add(C.X, sub(b, c));
+            C.Y = add(C.Y, sub(d, e));
+        }
+        F2 yp, ym, xyp, xym, yxp, yxm;
+        if (y0 || yN || edge) {
+            pair(n, n.v, false, yp, ym);
+            pair(n, add(n.u, n.v), true, xyp, xym);  // (1,1,0) (-1,-1,0)
+            pair(n, sub(n.u, n.v), true, yxp, yxm);  // (1,-1,0) (-1,1,0)
+        }
+        if (y0) {
+            const float b = z0 ? 0.f : yzm.x, c = zN ? 0.f : zym.x, s = ym.x + (xym.x + yxp.x) + (b + c);
+            C.D.x += s;
+            C.Y.x += s;
+            C.X.x += xym.x - yxp.x;
+            C.Z.x += b - c;
+        }
+        if (yN) {
+            const float w = dm.lid_axis == 1 ? dm.wall * (1.f / 36.f) : 0.f;
+            const float a = yp.y - 2.f * w * dm.lid[1];
+            const float b = yxm.y + w * (dm.lid[0] - dm.lid[1]), c = xyp.y + w * (-dm.lid[0] - dm.lid[1]);
+            const float d = z0 ? 0.f : zyp.y + w * (dm.lid[2] - dm.lid[1]);
+            const float e = zN ? 0.f : yzp.y + w * (-dm.lid[2] - dm.lid[1]);
+            const float s = a + (b + c) + (d + e);
+            C.D.y += s;
+            C.Y.y -= s;
+            C.X.y += b - c;
+            C.Z.y += d - e;
+        }
+        if (edge) {
+            F2 xp, xm;
+            pair(n, n.u, false, xp, xm);
+            if (e0 || eN) {
+                const F2 zero = bc<F2>(0.f), a = e0 ? xm : xp;
+                F2 b = e0 ? xzm : zxp, c = e0 ? zxm : xzp, d = e0 ? xym : yxp, e = e0 ? yxm : xyp;
+                if (z0) b = zero;
+                if (zN) c = zero;
+                if (y0) d.x = 0.f;
+                if (yN) e.y = 0.f;
+                const F2 s = add(a, add(add(b, c), add(d, e)));
+                C.D = add(C.D, s);
+                C.X = e0 ? add(C.X, s) : sub(C.X, s);
+                C.Z = add(C.Z, sub(b, c));
+                C.Y = add(C.Y, sub(d, e));
+            }
+        }
     }
     template <int MODE>
     __device__ __forceinline__ void receive(const Send &up, const Send &dn, Sum3 &P, Sum3 &C, Sum3 &N) const {
@@ -292,6 +391,10 @@ struct March3 {
         Sum3 N[2];
         in_row<MODE>(n0, d0, P[0], C[0], N[0], g[0][0], g[0][1], g[0][2]);
         in_row<MODE>(n1, d1, P[1], C[1], N[1], g[1][0], g[1][1], g[1][2]);
+        if (WALLS && (MODE == START || MODE == MID)) {
+            bounce(n0, 0, z, C[0]);
+            bounce(n1, 1, z, C[1]);
+        }
         Send up0, dn0, up1, dn1, h;
         halo<MODE>(nh, h);
         to_rows<MODE>(n0, up0, dn0);
@@ -315,8 +418,15 @@ struct March3 {
     __device__ __forceinline__ void planes(int za, int zb) const {
         Raw r;
         Sum3 pa[2], pb[2];
-        load(za - 1, r);
-        source<FIRST>(za - 1, r, pa, pb, true);
+        const bool floor = WALLS && dm.wz && za == 0, roof = WALLS && dm.wz && zb == dm.nz;
+        if (floor) {  // nothing comes through a z wall
+#pragma unroll
+            for (int p = 0; p < 2; ++p) pa[p].D = pa[p].X = pa[p].Y = bc<F2>(0.f);
+            load(za, r);
+        } else {
+            load(za - 1, r);
+            source<FIRST>(za - 1, r, pa, pb, true);
+        }
         source<START>(za, r, pb, pa, true);
         int z = za + 1;
         for (; z + 1 < zb; z += 2) {
@@ -325,7 +435,12 @@ struct March3 {
         }
         if (z < zb) {
             source<MID>(z, r, pa, pb, true);
-            source<LAST>(z + 1, r, pb, pa, false);
+            if (roof)
+                finish(z, pb);
+            else
+                source<LAST>(z + 1, r, pb, pa, false);
+        } else if (roof) {
+            finish(z - 1, pa);
         } else {
             source<LAST>(z, r, pa, pb, false);
         }
@@ -335,7 +450,7 @@ struct March3 {
 // items numbered strips first, then groups of kWarps tiles, then runs of planes, so that
 // the neighbours of a strip pass each plane together and share its lines in L2 (runs of
 // equal length that cross from column to column, out of step, took 235 us on 256^3)
-template <typename T, bool FIELD>
+template <typename T, bool FIELD, bool WALLS>
 __global__ void __launch_bounds__(32 * kWarps) k_d3q19_rows(const T *__restrict__ in, T *__restrict__ out, Dom3 dm,
                                                             int strips, int groups, int runs) {
     // the next step's CTAs may take their SMs as this step's leave them; none touches
@@ -347,18 +462,18 @@ __global__ void __launch_bounds__(32 * kWarps) k_d3q19_rows(const T *__restrict_
     if (y0 >= dm.ny) return;
     // the last tile ends with the domain: rows that two tiles update get the same values twice
     y0 = min(y0, dm.ny - kTile);
-    const March3<T, FIELD> m(in, out, dm, strip * kStrip, y0);
+    const March3<T, FIELD, WALLS> m(in, out, dm, strip * kStrip, y0);
     asm volatile("griddepcontrol.wait;" ::: "memory");
     m.planes((int)((long long)dm.nz * run / runs), (int)((long long)dm.nz * (run + 1) / runs));
 }
 
 // CTAs of the kernel that the GPU holds (-1 when it cannot be determined)
-template <typename T, bool FIELD>
+template <typename T, bool FIELD, bool WALLS>
 int room() {
     static DevSlots cap;
     return per_device(cap, [] {
         int per = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_d3q19_rows<T, FIELD>, 32 * kWarps, 0) !=
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_d3q19_rows<T, FIELD, WALLS>, 32 * kWarps, 0) !=
                 cudaSuccess || per < 1)
             return -1;
         return per * device_sms();
@@ -383,7 +498,7 @@ int plan_runs(long long cols, int nz, int room) {
     return best;
 }
 
-template <typename T, bool FIELD>
+template <typename T, bool FIELD, bool WALLS>
 cudaError_t launch_t(const void *in, void *out, const Dom3 &dm, int strips, int groups, int runs, cudaStream_t st) {
     const long long ctas = (long long)strips * groups * runs;
     if (ctas > 0x7fffffffLL) return cudaErrorInvalidValue;
@@ -396,12 +511,12 @@ cudaError_t launch_t(const void *in, void *out, const Dom3 &dm, int strips, int 
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_d3q19_rows<T, FIELD>, (const T *)in, (T *)out, dm, strips, groups, runs);
+    return cudaLaunchKernelEx(&cfg, k_d3q19_rows<T, FIELD, WALLS>, (const T *)in, (T *)out, dm, strips, groups, runs);
 }
 
-template <typename T, bool FIELD>
+template <typename T, bool FIELD, bool WALLS>
 cudaError_t launch_t(const void *in, void *out, const StepParams &p, cudaStream_t st) {
-    const int places = room<T, FIELD>();
+    const int places = room<T, FIELD, WALLS>();
     if (places < 1) return cudaErrorNotSupported;
     Dom3 dm;
     dm.nx = p.nx;
@@ -414,8 +529,14 @@ cudaError_t launch_t(const void *in, void *out, const StepParams &p, cudaStream_
     for (int c = 0; c < 3; ++c) dm.g[c] = p.has_force ? p.force[c] : 0.f;
     dm.forced = p.has_force || p.gfield;
     dm.field = p.gfield;
+    dm.wx = p.walled[0];
+    dm.wy = p.walled[1];
+    dm.wz = p.walled[2];
+    dm.lid_axis = p.lid_axis;
+    dm.wall = p.wallc;
+    for (int c = 0; c < 3; ++c) dm.lid[c] = p.lid[c];
     const int strips = (p.nx - 1) / kStrip + 1, groups = (p.ny - 1) / (kTile * kWarps) + 1;
-    return launch_t<T, FIELD>(in, out, dm, strips, groups, plan_runs((long long)strips * groups, p.nz, places), st);
+    return launch_t<T, FIELD, WALLS>(in, out, dm, strips, groups, plan_runs((long long)strips * groups, p.nz, places), st);
 }
 
 }  // namespace
@@ -425,12 +546,25 @@ bool rows3d_supported(const StepParams &p) {
     return p.ny >= kTile && (long long)p.nx * p.ny < (1LL << 30) && p.sdelta == 0.f && !p.scalar && !p.bulk;
 }
 
+// Walls applied in the kernel (no wall pass after it), without a force field, up to 2^20 nodes:
+// the bounces take registers (232: two CTAs a SM instead of four) and instructions in every
+// boundary warp, a wall pass 5 to 8 us a step (kernel and pass / walls in the kernel: the 60^3
+// cavity 9.7 / 5.2, 125 x 74 x 37 11.1 / 8.1, 100^3 18.6 / 18.1, 200^3 81 / 104).
+bool rows3d_walls(const StepParams &p) {
+    return p.bc != BC_PERIODIC && !p.gfield && p.N <= (1LL << 20) && rows3d_supported(p);
+}
+
+template <typename T>
+static cudaError_t rows3d_t(const void *in, void *out, const StepParams &p, cudaStream_t st) {
+    if (p.gfield) return launch_t<T, true, false>(in, out, p, st);
+    return rows3d_walls(p) ? launch_t<T, false, true>(in, out, p, st) : launch_t<T, false, false>(in, out, p, st);
+}
+
 cudaError_t launch_step_rows3d(int storage, const void *in, void *out, const StepParams &p, cudaStream_t st) {
     switch (storage) {
-        case STORE_F32: return p.gfield ? launch_t<float, true>(in, out, p, st) : launch_t<float, false>(in, out, p, st);
-        case STORE_BF16:
-            return p.gfield ? launch_t<__nv_bfloat16, true>(in, out, p, st) : launch_t<__nv_bfloat16, false>(in, out, p, st);
-        case STORE_F16: return p.gfield ? launch_t<__half, true>(in, out, p, st) : launch_t<__half, false>(in, out, p, st);
+        case STORE_F32: return rows3d_t<float>(in, out, p, st);
+        case STORE_BF16: return rows3d_t<__nv_bfloat16>(in, out, p, st);
+        case STORE_F16: return rows3d_t<__half>(in, out, p, st);
     }
     return cudaErrorInvalidValue;
 }

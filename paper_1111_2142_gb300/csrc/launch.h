@@ -101,6 +101,7 @@ bool cluster2d_supported(const StepParams &p);
 cudaError_t launch_cluster2d(int storage, const void *in, void *out, const StepParams &p, int steps, cudaStream_t st);
 // the plain D3Q19 scheme by warps that march along z (kernels_rows3.cu), any size
 bool rows3d_supported(const StepParams &p);
+bool rows3d_walls(const StepParams &p);  // whether it applies the walls itself
 cudaError_t launch_step_rows3d(int storage, const void *in, void *out, const StepParams &p, cudaStream_t st);
 cudaError_t launch_batch_step(int Q, int storage, const void *in, void *out, const BatchParams &bp,
                               cudaStream_t st);

@@ -336,9 +336,10 @@ cudaError_t step_between(lwacm_ctx *c, const void *in, void *out, cudaStream_t s
                     : c->kernel == 6 ? launch_step_tiles2d(c->Q, c->storage, c->batch_shape, in, out, p, st)
                                      : launch_step_generic(c->Q, c->storage, in, out, p, st);
     if (e != cudaSuccess) return e;
-    // the 2D-tile kernel applies the wall rule itself; the half-row kernel the x-face
-    // walls of a cavity whose lid is not on an x face
-    if (c->bc != LWACM_BC_PERIODIC && c->kernel != 6) {
+    // the D2Q9 and the marching D3Q19 kernels apply the wall rule themselves; the half-row
+    // kernel the x-face walls of a cavity whose lid is not on an x face
+    const bool walls_done = c->kernel == 6 || ((c->march || c->kernel == 1) && c->Q == 19 && rows3d_walls(p));
+    if (c->bc != LWACM_BC_PERIODIC && !walls_done) {
         StepParams pw = p;
         pw.xfaces_done = c->kernel == 5 && !c->march && half_xwalls(p) ? 1 : 0;
         e = launch_wall_pass(c->Q, c->storage, in, out, pw, st);

@@ -24,9 +24,9 @@ def lw():
     return lwacm
 
 
-def run(lw, shape, f, T, g=None, nu_p=None, **kw):
+def run(lw, shape, f, T, g=None, nu_p=None, bc=0, **kw):
     nz, ny, nx = shape
-    sim = lw.Lwacm(19, nx, ny, nz, 0.02, force_field=g is not None, kernel=1, **kw)
+    sim = lw.Lwacm(19, nx, ny, nz, 0.02, bc, force_field=g is not None, kernel=1, **kw)
     if nu_p:
         sim.set_option(lw.OPT_NU_P, nu_p)
     sim.set_fields(*f)
@@ -48,6 +48,19 @@ def within(got, ref, U=0.05):
 def test_march_matches_oracle(lw, shape):
     f = inputs.smooth_random(shape, seed=51, u_amp=0.05, d_amp=0.01)
     within(run(lw, shape, f, 9), oracle.step(19, *f, nu=0.02, nsteps=9))
+
+
+# walls in the kernel: two nodes an axis, strips and tiles that are at both walls, at one, at
+# none, tiles that overlap at the wall, several runs of planes
+@pytest.mark.parametrize("bc", [1, 2])
+@pytest.mark.parametrize("shape", [(2, 4, 2), (2, 5, 3), (3, 6, 29), (4, 7, 30), (5, 9, 31), (3, 8, 61), (6, 33, 95), (61, 66, 70)])
+def test_march_with_walls(lw, shape, bc):
+    """A cavity whose lid moves along all three axes' directions in the top z plane, and a
+    forced channel with a moving wall."""
+    f = inputs.smooth_random(shape, seed=56, u_amp=0.05, d_amp=0.01)
+    lid, force = (0.05, -0.03, 0.01), (1e-5, 0.0, 2e-5) if bc == 2 else None
+    got = run(lw, shape, f, 12, bc=bc, lid=lid, force=force)
+    within(got, oracle.step(19, *f, nu=0.02, nsteps=12, bc=bc, lid=lid, force=force))
 
 
 @pytest.mark.parametrize("shape", [(1, 4, 1), (2, 17, 61), (5, 15, 33)])
