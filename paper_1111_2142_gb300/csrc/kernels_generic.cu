@@ -482,21 +482,43 @@ __global__ void k_to_f32(const T *__restrict__ in, float *__restrict__ out, long
         out[i] = ldf(in + i);
 }
 template <typename Ti, typename T>
-__global__ void k_from(const Ti *__restrict__ in, T *__restrict__ out, long long n) {
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x) {
-        if constexpr (sizeof(Ti) == 8) {
-            // round once from FP64 to the storage type
-            if constexpr (sizeof(T) == 4)
-                out[i] = __double2float_rn(in[i]);
-            else if constexpr (std::is_same<T, __half>::value)
-                out[i] = __double2half(in[i]);
-            else
-                out[i] = __double2bfloat16(in[i]);
-        } else {
-            stf(out + i, in[i]);
+__device__ __forceinline__ T rounded(Ti v) {
+    if constexpr (sizeof(Ti) == 8) {
+        // round once from FP64 to the storage type
+        if constexpr (sizeof(T) == 4)
+            return __double2float_rn(v);
+        else if constexpr (std::is_same<T, __half>::value)
+            return __double2half(v);
+        else
+            return __double2bfloat16(v);
+    } else {
+        T t;
+        stf(&t, v);
+        return t;
+    }
+}
+// the fields of a state (or of a force) in one launch, blockIdx.y the field: a launch a field
+// cost a small domain more than its step (64^2: three launches 7 us, now 2.5)
+struct Sources {
+    const void *p[4];
+};
+template <typename Ti, typename T>
+__global__ void k_from(Sources src, T *__restrict__ dst, long long stride, long long n) {
+    const int f = (int)blockIdx.y;
+    const Ti *__restrict__ in = (const Ti *)(f == 0 ? src.p[0] : (f == 1 ? src.p[1] : (f == 2 ? src.p[2] : src.p[3])));
+    T *__restrict__ out = dst + blockIdx.y * stride;
+    const long long t0 = (long long)blockIdx.x * blockDim.x + threadIdx.x, step = (long long)gridDim.x * blockDim.x;
+    if constexpr (sizeof(Ti) == 4) {
+        if ((reinterpret_cast<uintptr_t>(in) & 15) == 0 && (reinterpret_cast<uintptr_t>(out) & 15) == 0) {
+            for (long long i = t0; i < n / 4; i += step) {
+                const float4 v = __ldg(reinterpret_cast<const float4 *>(in) + i);
+                tile::st4(out + 4 * i, v.x, v.y, v.z, v.w);
+            }
+            for (long long i = n / 4 * 4 + t0; i < n; i += step) out[i] = rounded<Ti, T>(in[i]);
+            return;
         }
     }
+    for (long long i = t0; i < n; i += step) out[i] = rounded<Ti, T>(in[i]);
 }
 
 // ---- FP64 diagnostics: per-block partials, then one block in fixed order ------
@@ -817,22 +839,30 @@ static unsigned conv_blocks(long long n) {
 }
 
 template <typename T>
-static cudaError_t from_t(int src_dtype, const void *src, void *dst, long long n, cudaStream_t st) {
+static cudaError_t from_t(int src_dtype, const Sources &src, int nf, void *dst, long long stride, long long n,
+                          cudaStream_t st) {
+    const dim3 grid(conv_blocks(n), (unsigned)nf);
     if (src_dtype == XFER_F64)
-        k_from<double, T><<<conv_blocks(n), 256, 0, st>>>((const double *)src, (T *)dst, n);
+        k_from<double, T><<<grid, 256, 0, st>>>(src, (T *)dst, stride, n);
     else
-        k_from<float, T><<<conv_blocks(n), 256, 0, st>>>((const float *)src, (T *)dst, n);
+        k_from<float, T><<<grid, 256, 0, st>>>(src, (T *)dst, stride, n);
     return cudaGetLastError();
 }
 
-cudaError_t launch_convert_in(int storage, int src_dtype, const void *src, void *dst, long long n,
-                              cudaStream_t st) {
+cudaError_t launch_convert_in_fields(int storage, int src_dtype, const void *const *src, int nf, void *dst,
+                                     long long stride, long long n, cudaStream_t st) {
+    Sources s = {};
+    for (int f = 0; f < nf; ++f) s.p[f] = src[f];
     switch (storage) {
-        case STORE_F32: return from_t<float>(src_dtype, src, dst, n, st);
-        case STORE_BF16: return from_t<__nv_bfloat16>(src_dtype, src, dst, n, st);
-        case STORE_F16: return from_t<__half>(src_dtype, src, dst, n, st);
+        case STORE_F32: return from_t<float>(src_dtype, s, nf, dst, stride, n, st);
+        case STORE_BF16: return from_t<__nv_bfloat16>(src_dtype, s, nf, dst, stride, n, st);
+        case STORE_F16: return from_t<__half>(src_dtype, s, nf, dst, stride, n, st);
     }
     return cudaErrorInvalidValue;
+}
+cudaError_t launch_convert_in(int storage, int src_dtype, const void *src, void *dst, long long n,
+                              cudaStream_t st) {
+    return launch_convert_in_fields(storage, src_dtype, &src, 1, dst, 0, n, st);
 }
 
 template <typename T>

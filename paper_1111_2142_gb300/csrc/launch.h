@@ -25,6 +25,9 @@ cudaError_t launch_semi_implicit(int Q, int storage, const void *in, void *out, 
                                  cudaStream_t st);
 cudaError_t launch_convert_in(int storage, int src_dtype, const void *src, void *dst, long long n,
                               cudaStream_t st);
+// nf (at most four) arrays on the device, array f to dst + f stride
+cudaError_t launch_convert_in_fields(int storage, int src_dtype, const void *const *src, int nf, void *dst,
+                                     long long stride, long long n, cudaStream_t st);
 cudaError_t launch_convert_out(int storage, int dst_dtype, const void *src, void *dst, long long n,
                                cudaStream_t st);
 cudaError_t launch_diagnostics(int storage, const void *f, long long fstride, long long N,

@@ -828,19 +828,16 @@ lwacm_status lwacm_set_fields(lwacm_ctx *c, const void *d, const void *ux, const
     const size_t nbytes = (size_t)c->N * sb;
     c->cur = 0;
     char *dst = (char *)bufp(c, 0);
-    for (int f = 0; f < c->nf; ++f) {
+    if (where == LWACM_DEVICE)
+        CK(c, launch_convert_in_fields(c->storage, dtype, src, c->nf, dst, c->Nal, c->N, c->stream), "convert in");
+    for (int f = 0; f < c->nf && where == LWACM_HOST; ++f) {
         char *fd = dst + (size_t)f * field_bytes(c);
         if (where == LWACM_HOST && dtype == LWACM_F32 && c->storage == LWACM_F32) {
             CK(c, cudaMemcpyAsync(fd, src[f], nbytes, cudaMemcpyHostToDevice, c->stream), "H2D");
             continue;
         }
-        const void *dsrc = src[f];
-        if (where == LWACM_HOST) {
-            CK(c, cudaMemcpyAsync(c->ws + c->off_stage, src[f], nbytes, cudaMemcpyHostToDevice, c->stream),
-               "H2D stage");
-            dsrc = c->ws + c->off_stage;
-        }
-        CK(c, launch_convert_in(c->storage, dtype, dsrc, fd, c->N, c->stream), "convert in");
+        CK(c, cudaMemcpyAsync(c->ws + c->off_stage, src[f], nbytes, cudaMemcpyHostToDevice, c->stream), "H2D stage");
+        CK(c, launch_convert_in(c->storage, dtype, c->ws + c->off_stage, fd, c->N, c->stream), "convert in");
     }
     // the scalar starts at zero until lwacm_set_scalar; the trace deviation of the
     // bulk-viscosity variant at zero (Tr^(+) = Tr^(e): the first step is the standard one)
@@ -870,22 +867,18 @@ lwacm_status lwacm_set_force_field(lwacm_ctx *c, const void *gx, const void *gy,
     const void *src[3] = {gx, gy, gz};
     const size_t sb = dtype == LWACM_F64 ? 8 : 4;
     const size_t nbytes = (size_t)c->N * sb;
-    for (int a = 0; a < c->D; ++a) {
+    if (where == LWACM_DEVICE)
+        CK(c, launch_convert_in_fields(STORE_F32, dtype, src, c->D, c->ws + c->off_ff, c->Nal, c->N, c->stream),
+           "force field copy");
+    for (int a = 0; a < c->D && where == LWACM_HOST; ++a) {
         char *dst = c->ws + c->off_ff + (size_t)a * c->Nal * 4;
         if (dtype == LWACM_F32) {
-            CK(c, cudaMemcpyAsync(dst, src[a], nbytes,
-                                  where == LWACM_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice,
-                                  c->stream),
-               "force field copy");
+            CK(c, cudaMemcpyAsync(dst, src[a], nbytes, cudaMemcpyHostToDevice, c->stream), "force field copy");
             continue;
         }
-        const void *dsrc = src[a];
-        if (where == LWACM_HOST) {
-            CK(c, cudaMemcpyAsync(c->ws + c->off_stage, src[a], nbytes, cudaMemcpyHostToDevice, c->stream),
-               "H2D stage");
-            dsrc = c->ws + c->off_stage;
-        }
-        CK(c, launch_convert_in(STORE_F32, LWACM_F64, dsrc, dst, c->N, c->stream), "force field convert");
+        CK(c, cudaMemcpyAsync(c->ws + c->off_stage, src[a], nbytes, cudaMemcpyHostToDevice, c->stream), "H2D stage");
+        CK(c, launch_convert_in(STORE_F32, LWACM_F64, c->ws + c->off_stage, dst, c->N, c->stream),
+           "force field convert");
     }
     if (!c->ff_active) {
         c->ff_active = true;
@@ -1166,8 +1159,7 @@ lwacm_status lwacm_backward(lwacm_ctx *c, const void *ld, const void *lux, const
     double *part = (double *)(A + L.part), *total = (double *)(A + L.total);
     unsigned *done = (unsigned *)(A + L.total + 8);
     const void *lin[4] = {ld, lux, luy, luz};
-    for (int f = 0; f < c->nf; ++f)
-        CK(c, launch_convert_in(STORE_F32, dtype, lin[f], (char *)lam0 + f * fb, c->N, c->stream), "lambda in");
+    CK(c, launch_convert_in_fields(STORE_F32, dtype, lin, c->nf, lam0, c->Nal, c->N, c->stream), "lambda in");
     CK(c, cudaMemsetAsync(total, 0, 16, c->stream), "clear dnu");
     const StepParams p = params(c);
     int cur = 0;

@@ -224,7 +224,7 @@ class Lwacm:
             keep = [np.ascontiguousarray(a, dtype=np.float64).reshape(-1) for a in arrs]
             dtype, where = F64, HOST
         else:
-            keep = [a.contiguous().reshape(-1) for a in arrs]
+            keep = [a.contiguous() for a in arrs]
             dt = keep[0].dtype
             dtype = {torch.float32: F32, torch.float64: F64}[dt]
             where = DEVICE if keep[0].is_cuda else HOST
@@ -250,7 +250,7 @@ class Lwacm:
             dtype, where = F64, HOST
         else:
             torch = _torch()
-            keep = [a.contiguous().reshape(-1) for a in arrs]
+            keep = [a.contiguous() for a in arrs]
             dtype = {torch.float32: F32, torch.float64: F64}[keep[0].dtype]
             where = DEVICE if keep[0].is_cuda else HOST
         for a in keep:

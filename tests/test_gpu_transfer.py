@@ -1,0 +1,55 @@
+"""Fields and forces copied in by one launch for all arrays: vector and single loads (aligned
+and unaligned sources, counts that are no multiple of four), every type."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def lw():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("needs a GPU")
+    from paper_1111_2142_gb300 import lwacm
+    return lwacm
+
+
+@pytest.mark.parametrize("dtype", ["float32", "float64"])
+@pytest.mark.parametrize("storage", [0, 1, 2])
+@pytest.mark.parametrize("shape", [(1, 1, 1), (1, 1, 3), (3, 5, 7), (4, 8, 64), (33, 65, 129)])
+@pytest.mark.parametrize("shift", [0, 1])
+def test_fields_from_device_arrays(lw, shape, storage, dtype, shift):
+    """The stored values are those of the same arrays handed over as FP64 host arrays (one copy
+    and one launch an array), the sources at 16-byte boundaries or one element past them."""
+    import torch
+    n = int(np.prod(shape))
+    g = torch.Generator(device="cuda").manual_seed(81)
+    f = [(torch.randn(n + shift, generator=g, device="cuda", dtype=getattr(torch, dtype)) * 0.05)[shift:].view(shape)
+         for _ in range(4)]
+    sim = lw.Lwacm(19, shape[2], shape[1], shape[0], 0.02, storage=storage)
+    sim.set_fields(*f)
+    got = [v.clone() for v in sim.fields()]
+    sim.set_fields(*[a.double().cpu().numpy() for a in f])
+    for a, v in zip(got, sim.fields()):
+        assert torch.equal(a, v)
+    sim.close()
+
+
+@pytest.mark.parametrize("dtype", ["float32", "float64"])
+def test_force_field_from_unaligned_arrays(lw, dtype):
+    """A force field from arrays one element past a 16-byte boundary acts as from aligned ones."""
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(82)
+    flat = [torch.randn(35 * 27 + 1, generator=g, device="cuda", dtype=getattr(torch, dtype)) * 1e-4 for _ in range(2)]
+    out = []
+    for a in ([t[1:].view(27, 35) for t in flat], [t[1:].view(27, 35).clone() for t in flat]):
+        sim = lw.Lwacm(9, 35, 27, 1, 0.02, force_field=True)
+        sim.set_fields(*[np.zeros((27, 35))] * 3)
+        sim.set_force_field(*a)
+        sim.step(3)
+        out.append(sim.get_fields())
+        sim.close()
+    for x, y in zip(*out):
+        assert np.array_equal(x, y)
+    assert float(np.max(np.abs(out[0][1]))) > 1e-5
