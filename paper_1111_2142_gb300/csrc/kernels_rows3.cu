@@ -541,6 +541,8 @@ cudaError_t launch_t(const void *in, void *out, const StepParams &p, cudaStream_
 
 }  // namespace
 
+int rows3d_runs(long long cols, int nz, int room) { return plan_runs(cols, nz, room); }
+
 bool rows3d_supported(const StepParams &p) {
     // a whole tile; a byte offset within a plane fits 32 bits; the plain scheme
     return p.ny >= kTile && (long long)p.nx * p.ny < (1LL << 30) && p.sdelta == 0.f && !p.scalar && !p.bulk;

@@ -104,6 +104,11 @@ bool cluster2d_supported(const StepParams &p);
 cudaError_t launch_cluster2d(int storage, const void *in, void *out, const StepParams &p, int steps, cudaStream_t st);
 // the plain D3Q19 scheme by warps that march along z (kernels_rows3.cu), any size
 bool rows3d_supported(const StepParams &p);
+// runs of planes a column of strips and tiles is cut into, for a GPU that holds `room` CTAs
+int rows3d_runs(long long cols, int nz, int room);
+// the passive scalar (Eq. ACM2.0t) the same way (kernels_scalar3.cu), after the flow kernel on the
+// same state; periodic, where rows3d_supported() but for the scalar
+cudaError_t launch_scalar_march(int storage, const void *in, void *out, const StepParams &p, cudaStream_t st);
 bool rows3d_walls(const StepParams &p);  // whether it applies the walls itself
 cudaError_t launch_step_rows3d(int storage, const void *in, void *out, const StepParams &p, cudaStream_t st);
 cudaError_t launch_batch_step(int Q, int storage, const void *in, void *out, const BatchParams &bp,

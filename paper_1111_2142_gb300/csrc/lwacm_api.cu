@@ -44,6 +44,7 @@ struct lwacm_ctx {
     bool no_cluster = false;  // the device does not take the cluster kernel
     bool march = false;       // kernel 5, automatic choice: by warps that march along z (kernels_rows3.cu)
     bool scalar_rows = false; // the passive scalar on its own row-tiled kernel after the flow kernel
+    bool scalar_march = false;  // on its own marching kernel after the general flow kernel
     int nsc = 0;              // fields stored after the flow fields: the scalar or the trace (0 or 1)
     long long N = 0, Nal = 0;
     double lid[3] = {0, 0, 0}, force[3] = {0, 0, 0}, rho0 = 1.0;
@@ -233,6 +234,9 @@ bool choose_kernel(lwacm_ctx *c) {
     static const char *sname[7] = {"tiles2d_d2q9_30x14", "tiles2d_d2q9_30x6",  "tiles2d_d2q9_30x14", "tiles2d_d2q9_62x6",
                                    "tiles2d_d2q9_30x30", "tiles2d_d2q9_62x14", "tiles2d_d2q9_126x6"};
     if (c->kernel != 5) c->scalar_rows = false;
+    StepParams flow = p;
+    flow.scalar = 0;
+    c->scalar_march = p.scalar && c->Q == 19 && c->kernel == 1 && rows3d_supported(flow);
     // rows the half-row kernel takes, plain scheme: marching warps, which need no halves or
     // segments (us a step, half-row / march: 256^3 137 / 129, 256 x 128 x 128 39 / 35, 384 x 256 x
     // 256 278 / 178, 200 x 256 x 256 190 / 100), but for whole rows of one warp (128 x 256 x 256 65 /
@@ -326,7 +330,7 @@ cudaError_t step_between(lwacm_ctx *c, const void *in, void *out, cudaStream_t s
     if (c->nbatch) return launch_batch_step(c->Q, c->storage, in, out, batch_params(c), st);
     const StepParams p = params(c);
     StepParams pf = p;
-    if (c->scalar_rows) pf.scalar = 0;  // the flow kernel leaves the scalar to its own kernel
+    if (c->scalar_rows || c->scalar_march) pf.scalar = 0;  // the flow kernel leaves the scalar to its own kernel
     cudaError_t e = cudaSuccess;
     if (c->kernel == 5 && p.sdelta != 0.f) e = launch_nup_sum(c->storage, in, p.nup_p, p, st);
     if (e != cudaSuccess) return e;
@@ -334,7 +338,7 @@ cudaError_t step_between(lwacm_ctx *c, const void *in, void *out, cudaStream_t s
                     : c->kernel == 5 ? launch_step_half(c->Q, c->storage, in, out, pf, st)
                     : c->kernel == 6 && c->batch_shape == 0 ? launch_step_rows2d(c->storage, in, out, p, st)
                     : c->kernel == 6 ? launch_step_tiles2d(c->Q, c->storage, c->batch_shape, in, out, p, st)
-                                     : launch_step_generic(c->Q, c->storage, in, out, p, st);
+                                     : launch_step_generic(c->Q, c->storage, in, out, pf, st);
     if (e != cudaSuccess) return e;
     // the D2Q9 and the marching D3Q19 kernels apply the wall rule themselves; the half-row
     // kernel the x-face walls of a cavity whose lid is not on an x face
@@ -346,7 +350,10 @@ cudaError_t step_between(lwacm_ctx *c, const void *in, void *out, cudaStream_t s
     }
     if (e == cudaSuccess && p.sr_ctr && c->kernel == 5) e = launch_sr_tick(p.sr_ctr, st);
     if (e == cudaSuccess && c->semi) e = launch_semi_implicit(c->Q, c->storage, in, out, p, st);
-    if (e == cudaSuccess && c->scalar_rows) e = launch_scalar_rows(in, out, p, st);
+    // rows of 128 nodes (one warp a row) on the row-tiled kernel, others by marching warps (us a step
+    // with the flow: 128 x 256 x 256 111.9 / 116.9, 256 x 256 x 128 125.1 / 120.5)
+    if (e == cudaSuccess && c->scalar_rows && c->nx == 128) e = launch_scalar_rows(in, out, p, st);
+    else if (e == cudaSuccess && (c->scalar_rows || c->scalar_march)) e = launch_scalar_march(c->storage, in, out, p, st);
     return e;
 }
 
