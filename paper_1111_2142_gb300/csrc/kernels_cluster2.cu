@@ -10,6 +10,9 @@
 // between. The barrier is the hardware's, and every thread of every CTA takes part in it the
 // same number of times.
 //
+// A thread reads its own nodes' fields at the start and writes them at the end, so `in` and
+// `out` may be one buffer.
+//
 // The values and sums are formed as the marching kernel forms them (rows2.cuh), in the same
 // order, so the fields do not depend on how many steps a launch takes (the bulk-viscosity
 // variant as there, in the 2D-tile kernel's order).
@@ -59,8 +62,7 @@ __device__ __forceinline__ void cluster_barrier() {
 }
 
 template <int PER, typename T, bool WALLS, bool BULK, bool NUP>
-__global__ void __launch_bounds__(kThreads) k_d2q9_cluster(const T *__restrict__ in, T *__restrict__ out, Small2 p,
-                                                           int steps) {
+__global__ void __launch_bounds__(kThreads) k_d2q9_cluster(const T *in, T *out, Small2 p, int steps) {
     constexpr int NV = NUP ? 12 : 8;  // values a node leaves: links 1 to 8, then W_0 to W_3
     constexpr int NF = BULK ? 4 : 3;
     extern __shared__ float sm[];
@@ -93,10 +95,10 @@ __global__ void __launch_bounds__(kThreads) k_d2q9_cluster(const T *__restrict__
         const long long g = (long long)y[k] * p.nx + x;
         d[k] = u[k] = v[k] = tr[k] = 0.f;
         if (on[k]) {
-            d[k] = ldf(in + g);
-            u[k] = ldf(in + p.fstride + g);
-            v[k] = ldf(in + 2 * p.fstride + g);
-            if (BULK) tr[k] = ldf(in + (NF - 1) * p.fstride + g);
+            d[k] = rows2::widen(rows2::ldraw<true>(in + g));
+            u[k] = rows2::widen(rows2::ldraw<true>(in + p.fstride + g));
+            v[k] = rows2::widen(rows2::ldraw<true>(in + 2 * p.fstride + g));
+            if (BULK) tr[k] = rows2::widen(rows2::ldraw<true>(in + (NF - 1) * p.fstride + g));
         }
     }
     cluster_barrier();  // every CTA runs before any writes to its shared memory

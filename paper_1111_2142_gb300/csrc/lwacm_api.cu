@@ -933,13 +933,16 @@ lwacm_status lwacm_step(lwacm_ctx *c, long long n) {
     long long left = n;
     while (on_cluster(c, left)) {
         const int m = (int)std::min<long long>(left, 8192);  // a launch of a few milliseconds
-        const cudaError_t e = launch_cluster2d(c->storage, bufp(c, c->cur), bufp(c, 1 - c->cur), params(c), m, c->stream);
+        // the state stays in its buffer after an even number of steps, as with single steps (a
+        // caller that captures an even number into a graph of its own replays it on and on)
+        const int to = c->cur ^ (m & 1);
+        const cudaError_t e = launch_cluster2d(c->storage, bufp(c, c->cur), bufp(c, to), params(c), m, c->stream);
         if (e != cudaSuccess) {  // refused before it ran (a device without clusters of this size)
             cudaGetLastError();
             c->no_cluster = true;
             break;
         }
-        c->cur ^= 1;
+        c->cur = to;
         c->steps += m;
         left -= m;
     }

@@ -70,3 +70,33 @@ def test_cluster_then_single_steps_and_long_runs(lw):
         sim.close()
     for a, b in zip(*out):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("n", [4, 5, 64])
+def test_cluster_leaves_the_state_in_the_buffer_of_single_steps(lw, n):
+    """An even number of steps ends in the buffer it started from, so that a caller's own graph
+    of them advances the state at every replay."""
+    import torch
+    f = inputs.smooth_random((20, 24), seed=73, u_amp=0.03, d_amp=0.005)
+    sim = lw.Lwacm(9, 24, 20, 1, 0.02, stream=torch.cuda.Stream())
+    sim.set_fields(*f)
+    before = sim.fields()[0].data_ptr()
+    sim.step(n)
+    assert (sim.fields()[0].data_ptr() == before) == (n % 2 == 0)
+    if n % 2 == 0:
+        sim.sync()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=sim.stream):
+            sim.step(n)
+        with torch.cuda.stream(sim.stream):
+            g.replay()
+            g.replay()
+        sim.sync()
+        ref = lw.Lwacm(9, 24, 20, 1, 0.02)
+        ref.set_fields(*f)
+        for _ in range(3 * n):
+            ref.step(1)
+        for a, b in zip(sim.get_fields(), ref.get_fields()):
+            assert np.array_equal(a, b)
+        ref.close()
+    sim.close()
