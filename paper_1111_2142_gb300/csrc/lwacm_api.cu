@@ -43,7 +43,7 @@ struct lwacm_ctx {
     bool sr = false;          // BF16 / FP16 stores rounded stochastically (half-row kernel)
     bool no_cluster = false;  // the device does not take the cluster kernel
     bool march = false;       // kernel 5, automatic choice: by warps that march along z (kernels_rows3.cu)
-    bool scalar_rows = false; // the passive scalar on its own row-tiled kernel after the flow kernel
+    bool scalar_rows = false; // the passive scalar on its own kernel after the half-row flow kernel
     bool scalar_march = false;  // on its own marching kernel after the general flow kernel
     int nsc = 0;              // fields stored after the flow fields: the scalar or the trace (0 or 1)
     long long N = 0, Nal = 0;
@@ -213,8 +213,8 @@ bool choose_kernel(lwacm_ctx *c) {
     }
     const StepParams p = params(c);
     const bool dev = c->bound;
-    // the passive scalar: on its own row-tiled kernel when the shape allows, the
-    // flow then on the half-row kernel; otherwise both on the generic kernel
+    // the passive scalar: on its own kernel, the flow on the half-row kernel when the shape
+    // allows, else by marching warps; both on the generic kernel with options those do not take
     c->scalar_rows = dev && p.scalar && scalar_rows_supported(c->Q, c->storage, p);
     StepParams pf = p;
     if (c->scalar_rows) pf.scalar = 0;
