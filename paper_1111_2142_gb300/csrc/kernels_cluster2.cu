@@ -74,7 +74,8 @@ __global__ void __launch_bounds__(kThreads) k_d2q9_cluster(const T *in, T *out, 
     const int pitch = (p.nrows + 2) * p.nx, set = NV * pitch;
     const uint32_t base = tile::sa(sm);
     const uint32_t base_up = map_rank(base, up), base_dn = map_rank(base, dn);
-    const float nu = p.s * (1.f / 18.f), am1 = p.s * (-1.f / 3.f), odd = p.s * (2.f / 9.f);
+    const float nu = p.s * (1.f / 18.f), odd = __fmul_rn(p.s, 2.f / 9.f);
+    const float am1 = BULK ? p.s * (-1.f / 3.f) : __fmul_rn(odd, -1.5f), am1l = fmaf(odd, -1.5f, -am1);  // as March's
     // the thread's nodes
     int at[PER], xl[PER], xr[PER];  // place in a value's array; the places of x - 1 and x + 1 less this one
     int y[PER], xs[PER];
@@ -174,7 +175,7 @@ __global__ void __launch_bounds__(kThreads) k_d2q9_cluster(const T *in, T *out, 
             float l5 = g(4, l - nx), r6 = g(5, r + nx), l7 = g(6, l + nx), r8 = g(7, r - nx);
             const float rho = __fadd_rn(d[k], 1.f);
             const float K = fmaf(__fmul_rn(rho, -1.5f), fmaf(u[k], u[k], __fmul_rn(v[k], v[k])), d[k]);
-            const float m = fmaf(p.a, d[k], am1);
+            const float m = BULK ? fmaf(p.a, d[k], am1) : __fadd_rn(fmaf(p.a, d[k], am1l), am1);
             float D, X, Y, un, vn, tn = 0.f;
             if (BULK) {
                 const float axs = __fadd_rn(__fadd_rn(l1, r2), __fadd_rn(g3, g4));

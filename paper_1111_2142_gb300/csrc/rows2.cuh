@@ -208,7 +208,10 @@ struct March {
     const Dom2 &dm;
     const Walls2 &wl;
     const Force2 &fc;
-    const float gamma, sdelta, nu, am1, odd;
+    // The links give a momentum j back 3/2 odd j and the post-combine 1 + am1 of it: 3/2 odd + am1
+    // has to vanish, or every step changes the momentum by the rest (rounded apart it was 6e-8 of
+    // 6 nu, 3e-7 of u after 24 steps at nu = 0.06), so am1 + am1l is -3/2 odd exactly
+    const float gamma, sdelta, nu, odd, am1, am1l;
     unsigned xo[NS];  // the lane's columns, wrapped
     bool st[NS], e0[NS], eN[NS];
     bool edge;  // the strips hold a column at an x wall
@@ -216,7 +219,8 @@ struct March {
     __device__ __forceinline__ March(const T *in_, T *out_, const Dom2 &dm_, int x0, const Walls2 &wl_,
                                      const Force2 &fc_, float gamma_, float sdelta_)
         : in(in_ + dm_.base), out(out_ + dm_.base), dm(dm_), wl(wl_), fc(fc_), gamma(gamma_), sdelta(sdelta_),
-          nu(dm_.s * (1.f / 18.f)), am1(dm_.s * (-1.f / 3.f)), odd(dm_.s * (2.f / 9.f)) {
+          nu(dm_.s * (1.f / 18.f)), odd(dm_.s * (2.f / 9.f)),
+          am1(BULK ? dm_.s * (-1.f / 3.f) : odd * -1.5f), am1l(fmaf(odd, -1.5f, -am1)) {
         const int lane = threadIdx.x & 31;
         edge = WALLS && wl.wx && (x0 == 0 || x0 + NS * kHalf >= dm.nx);
 #pragma unroll
@@ -331,7 +335,7 @@ struct March {
         if (OWN) {  // the row itself: rest and c_y = 0 links, and a rho u = u + m u (u added last)
             C.D = fma(4.f / 9.f, K, add(C.D, add(l1, r2)));
             if (NUP) C.S = add(C.S, sub(from_left(W[0]), from_right(W[0])));
-            const F m = fma(dm.a, d, bc<F>(am1));
+            const F m = add(fma(dm.a, d, bc<F>(am1l)), am1);
             C.X = fma(m, u, add(C.X, sub(l1, r2)));
             C.Y = fma(m, v, C.Y);
             if (WALLS && edge) {  // the diagonal links (in a row at a y wall the row beyond it has them)
