@@ -229,6 +229,7 @@ def _events_ms(stream, fn):
 
 KERNEL_SOURCES = {
     "half_d3q19_tma": ("kernels_half.cu", "tile_common.cuh", "lwacm_core.cuh"),
+    "half_d3q19_march": ("kernels_rows3.cu", "rows2.cuh", "tile_common.cuh", "lwacm_core.cuh"),
 }
 
 
@@ -277,7 +278,7 @@ def variants(hbm):
                      "hbm_frac": bpn * g / hbm, "bytes_per_node": bpn}
         sim.close()
         torch.cuda.empty_cache()
-    # rows longer than 256: the half-row kernel on 128-node segments, and the generic kernel
+    # rows longer than 256: the automatic choice, and the general kernel (both marching warps)
     sx, sy, sz = 384, 256, 256
     fs = inputs.tgv3d(sx, u0=U0, ny=sy, nz=sz)
     seg = {"shape": [sx, sy, sz], "unit": "GLUPS", "bytes_per_node": 32}
@@ -456,7 +457,7 @@ def next_rows(hbm, glups):
     t3 = torch.cos(2 * torch.pi * torch.arange(n3, device="cuda") / n3).expand(n3, n3, n3).contiguous()
     timed("scalar_d3q19_256", lw.Lwacm(lw.D3Q19, n3, n3, n3, NU, scalar_alpha=0.01), f3, 100, n3 ** 3, 40,
           extra=lambda s: s.set_scalar(t3))
-    # a constant acceleration (Eq. force) on the 256^3 Taylor-Green workload (half-row kernel)
+    # a constant acceleration (Eq. force) on the 256^3 Taylor-Green workload
     timed("forced_d3q19_256", lw.Lwacm(lw.D3Q19, n3, n3, n3, NU, force=(1e-6, 0.0, 0.0)), f3, 200, n3 ** 3, 32)
     # omega_p on the 256^3 Taylor-Green workload: the density-term pass (reads the state,
     # writes one FP32 field) and the half-row kernel (reads that field too): 52 B/node
@@ -667,7 +668,7 @@ def run_case(name, steps):
         sim = lw.Lwacm(lw.D3Q19, 256, 256, 256, 0.01, lw.CAVITY, lid=(2 ** 0.5 / 20, 2 ** 0.5 / 20, 0.0))
         sim.set_fields(z, z, z, z)
         sim.step(steps)
-    elif name == "scalar":  # D3Q19 256^3 Taylor-Green with a passive scalar (half-row + scalar row kernels)
+    elif name == "scalar":  # D3Q19 256^3 Taylor-Green with a passive scalar (half-row + marching scalar kernels)
         n3 = 256
         sim = lw.Lwacm(lw.D3Q19, n3, n3, n3, NU, scalar_alpha=0.01)
         sim.set_fields(*inputs.tgv3d(n3, u0=U0))
@@ -678,11 +679,11 @@ def run_case(name, steps):
         sim.set_option(lw.OPT_NU_P, 0.05)
         sim.set_fields(*inputs.tgv3d(256, u0=U0))
         sim.step(steps)
-    elif name == "segments":  # D3Q19 384 x 256 x 128 Taylor-Green (half-row kernel on 128-node segments)
+    elif name == "segments":  # D3Q19 384 x 256 x 128 Taylor-Green (marching warps)
         sim = lw.Lwacm(lw.D3Q19, 384, 256, 128, NU)
         sim.set_fields(*inputs.tgv3d(384, u0=U0, ny=256, nz=128))
         sim.step(steps)
-    elif name == "bulk2d":  # D2Q9 4096^2 bulk-viscosity variant, gamma 0.4 (2D tiles 30x14)
+    elif name == "bulk2d":  # D2Q9 4096^2 bulk-viscosity variant, gamma 0.4 (marching warps)
         sim = lw.Lwacm(lw.D2Q9, 4096, 4096, 1, 0.01, bulk_gamma=0.4)
         sim.set_fields(*inputs.gtg_state(4096, 0.0))
         sim.step(steps)

@@ -98,7 +98,7 @@ enum {
                               domains with the wall pass
                               after it; FP32, BF16 and FP16 storage: LWACM_E_UNSUPPORTED
                               otherwise); 2 and 3 (earlier row-tiled kernels, superseded
-                              by 5) are retired: LWACM_E_ARG; 6 = D2Q9 2D-tile kernel (any boundary, walls
+                              by 5) are retired: LWACM_E_ARG; 6 = D2Q9 kernels (any boundary, walls
                               and forcing applied in the kernel; omega_p and the
                               bulk-viscosity variant (alone or together) on periodic
                               domains; not the scalar; tile shape from
@@ -130,8 +130,9 @@ enum {
                                      i.e. omega_p of Section 2.2 item 3 (Eq. FDcompact c
                                      relaxed with omega_p, momentum with omega): in (0,
                                      1/6], or 0 = nu (default). Single periodic domains
-                                     only (LWACM_E_UNSUPPORTED otherwise); runs on the
-                                     D2Q9 2D-tile kernel, else on the generic kernel;
+                                     only (LWACM_E_UNSUPPORTED otherwise); runs on kernel 6
+                                     (D2Q9), on kernel 5 where it applies after a pass
+                                     that sums the density term, else on kernel 1;
                                      the adjoint refuses nu_p != nu. */
     LWACM_OPT_SCALAR_ALPHA = 15,  /* > 0: carry a passive scalar T (Eq. ACM2.0t, the
                                      thermal LW-ACM of Appendix "Asymptotic analysis for
@@ -140,7 +141,8 @@ enum {
                                      advected by the flow velocity at each step's time
                                      level; 0 = none (default). Before lwacm_bind (it
                                      adds one field to the workspace); single periodic
-                                     domains only; runs on the generic kernel. */
+                                     domains only. D3Q19 runs it on its own kernel after the
+                                     flow's, D2Q9 on kernel 1. */
     LWACM_OPT_BULK_GAMMA = 16,    /* gamma in (-1, 1), 0 = off (default): the bulk-
                                      viscosity variant of Appendix "Computing derivatives
                                      locally", Eq. quasi-equilibrium2. The equilibrium of
@@ -160,7 +162,7 @@ enum {
                                      periodic D2Q9 domains only, not with the scalar
                                      (LWACM_E_UNSUPPORTED). With LWACM_OPT_NU_P the density
                                      is relaxed with omega_p and the momentum and the
-                                     trace with omega. Runs on the D2Q9 2D-tile kernel. */
+                                     trace with omega. Runs on kernel 6. */
     LWACM_OPT_SEMI_IMPLICIT = 17, /* 1: semi-implicit pressure update (Section 2.2 item 2,
                                      Eq. FDcompact_si), 0 = explicit (default). The
                                      velocity is that of the explicit step; the density
@@ -245,10 +247,10 @@ lwacm_status lwacm_set_fields(lwacm_ctx *ctx, const void *d, const void *ux, con
  * the next call. The step adds rho(x,t) g(x) to the momentum, on top of any
  * constant LWACM_OPT_FORCE_* vector. All three pointers NULL switches the field
  * off. Stream-ordered on the bound stream (host buffers must stay valid until
- * the stream reaches this point; FP32 host arrays should be pinned). The D3Q19
- * row-tiled kernels have no forcing term, so a D3Q19 context with forcing runs
- * the generic kernel; D2Q9 runs the 2D-tile kernel, which adds it. The adjoint (lwacm_forward_record) refuses a context whose field is on
- * (LWACM_E_UNSUPPORTED).
+ * the stream reaches this point; FP32 host arrays should be pinned). The half-row
+ * kernel takes no field: a D3Q19 context with one runs kernel 1, whose marching warps add
+ * it; D2Q9 adds it in kernel 6. The adjoint (lwacm_forward_record) refuses a context
+ * whose field is on (LWACM_E_UNSUPPORTED).
  * Errors: LWACM_E_STATE (nothing reserved, or not bound), LWACM_E_ARG. */
 lwacm_status lwacm_set_force_field(lwacm_ctx *ctx, const void *gx, const void *gy, const void *gz,
                                    int dtype, int where);

@@ -1,6 +1,9 @@
 // Half-row TMA row-tiled D3Q19 kernel, for domains with nx = 256, 128 or other rows
-// of at least 72 nodes (multiples of 4, see segments_fit) and any ny (periodic; walled domains get the wall pass after it,
-// the cavity's x faces handled here for rows of 128 and 256): the moment form of
+// of at least 72 nodes (multiples of 4, see segments_fit) and any ny (periodic; walled
+// domains get the wall pass after it, the cavity's x faces handled here for rows of 128
+// and 256). The automatic choice takes it for rows of 128, such cavities, omega_p,
+// stochastic rounding and beside a scalar, elsewhere the marching warps of
+// kernels_rows3.cu are the faster ones. The moment form of
 // Eq. ACM2.0 (see lwacm_core.cuh), every field read from HBM once and written once
 // per step. A CTA updates columns of 8 rows; when ny % 8 != 0 the last column's
 // rows beyond ny hold the rows that follow it periodically, so its first such row
