@@ -57,7 +57,8 @@ __global__ void __launch_bounds__(256) k_adj_prep(const float *__restrict__ sn, 
 // where weighting each pair (c, -c) into the ten moments took six FMAs a pair. With it, the
 // overlapped launch (k_adj_rows) and one staged plane for D2Q9 a step of a 24-step sweep takes, us
 // before / after: 128^3 32.8 / 30.0, 256 x 128 x 64 37.7 / 35.5, 100 x 90 x 80 31.1 / 28.7,
-// 800 x 700 22.7 / 21.2. Bound by instructions, with two CTAs of eight warps a SM.
+// 800 x 700 22.7 / 21.2. k_adj_rows: 202 instructions a node (230
+// before), issue slots 49% busy with 16 warps a SM that wait on shared memory and the plane barrier.
 struct Corners {
     float t, a, b, ab;
 };

@@ -14,7 +14,7 @@
 // The loads of the next plane are in flight meanwhile.
 //
 // What bounds it, FP32 256^3 (128 GLUPS, 131 us a step): instructions, 153 a node (85 of them
-// FP32, most packed), issue slots 49% and the FMA pipe 59% busy with 16 warps a SM; DRAM 49%.
+// FP32, most packed), issue slots 51% and the FMA pipe 58% busy with 16 warps a SM; DRAM 47%.
 // Measured and left out: the next planes in a ring in shared memory by asynchronous copies
 // (no waits for memory, but 180 instructions a node: 138 us), 20 warps at 96 registers (135
 // us), 12 warps at 168 (141 us).
