@@ -52,34 +52,6 @@ __global__ void __launch_bounds__(256) k_adj_prep(const float *__restrict__ sn, 
     }
 }
 
-// The four diagonal links of a plane (a, b), gbar from the receivers at ++, -+, +-, -- : their sum
-// goes to G0, G2aa and G2bb, the differences to G1a, G1b and G2ab. Eight additions for all four,
-// where weighting each pair (c, -c) into the ten moments took six FMAs a pair. With it, the
-// overlapped launch (k_adj_rows) and one staged plane for D2Q9 a step of a 24-step sweep takes, us
-// before / after: 128^3 32.8 / 30.0, 256 x 128 x 64 37.7 / 35.5, 100 x 90 x 80 31.1 / 28.7,
-// 800 x 700 22.7 / 21.2. k_adj_rows: 202 instructions a node (230
-// before), issue slots 49% busy with 16 warps a SM that wait on shared memory and the plane barrier.
-struct Corners {
-    float t, a, b, ab;
-};
-__device__ __forceinline__ Corners corners(float pp, float mp, float pm, float mm) {
-    const float u = pp + mp, v = pm + mm, du = pp - mp, dv = pm - mm;
-    return Corners{u + v, du + dv, u - v, du - dv};
-}
-
-// the link of velocity (cx, cy, cz)
-template <int Q>
-__host__ __device__ constexpr int link_of(int cx, int cy, int cz) {
-    for (int i = 0; i < Q; ++i)
-        if (Lat<Q>::c(i, 0) == cx && Lat<Q>::c(i, 1) == cy && Lat<Q>::c(i, 2) == cz) return i;
-    return 0;
-}
-
-template <int Q, int CX, int CY, int CZ>
-struct Link {
-    static constexpr int value = link_of<Q>(CX, CY, CZ);
-};
-
 // lambda at t from (Dbar, Jbar) gathered at the downwind neighbours and the state
 // at t, with the (Dbar, Jbar) fields staged in shared memory: a CTA of
 // 32 x 8 threads takes an x-y tile of the domain and marches along z through a run
@@ -89,7 +61,7 @@ struct Link {
 // two planes earlier, so one barrier per plane orders it). The state at t of the
 // plane z+1 is loaded into registers while the plane z is computed.
 constexpr int ATX = 32, ATY = 8, AZC = 8;
-constexpr int AW = ATX + 2, AH = ATY + 2, APL = AW * AH;
+constexpr int AW = ATX + 2, AH = ATY + 2, APL = AW * AH, NSL = 5;
 
 // With WALLS, a link whose receiver x + c lies beyond a walled face is the value the
 // node itself takes for the bounced link -c (Eq. ACM2.0cccbb2): gbar = Dbar - c.Jbar
@@ -103,7 +75,7 @@ __global__ void __launch_bounds__(ATX *ATY) k_adj_gather_tiled(const float *__re
                                                                unsigned *__restrict__ done,
                                                                double *__restrict__ nu_total) {
     using L = Lat<Q>;
-    constexpr int NF = Q == 19 ? 4 : 3, NSL = Q == 19 ? 5 : 1;  // D2Q9: one plane, staged once
+    constexpr int NF = Q == 19 ? 4 : 3;
     __shared__ float ring[NSL][NF][APL];
     const int tid = (int)threadIdx.x, tx = tid % ATX, ty = tid / ATX;
     const long long plane = (long long)p.nx * p.ny;
@@ -160,12 +132,12 @@ __global__ void __launch_bounds__(ATX *ATY) k_adj_gather_tiled(const float *__re
             if (Q == 19) w = st[3 * p.fstride + k];
         }
         __syncthreads();  // the previous item's last reads are done
-        if (Q == 19) issue(za - 1);
+        issue(za - 1);
         issue(za);
-        if (Q == 19) issue(za + 1);
+        issue(za + 1);
         for (int z = za; z < zb; ++z) {
             // planes z-1, z, z+1 complete (z+2 may still be in flight)
-            if (Q == 19 && z + 2 <= zb) {
+            if (z + 2 <= zb) {
                 issue(z + 2);
                 asm volatile("cp.async.wait_group 1;" ::: "memory");
             } else {
@@ -190,8 +162,8 @@ __global__ void __launch_bounds__(ATX *ATY) k_adj_gather_tiled(const float *__re
                 //   sum_i gbar_i dg_i/dd = (1 - 3/2 q) G0 + s u.G1 + 9/2 u.G2.u,
                 //   sum_i gbar_i dg_i/du = rho (s G1 + 9 G2.u - 3 u G0),
                 //   sum_i gbar_i dg_i/ds = rho u.G1
-                // (below without the 1/36 of the diagonal links' weight)
-                float gbar[Q];
+                float g0 = 0.f, g1x = 0.f, g1y = 0.f, g1z = 0.f;
+                float gxx = 0.f, gyy = 0.f, gzz = 0.f, gxy = 0.f, gxz = 0.f, gyz = 0.f;
                 float nu_wall = 0.f;  // sum over lid links of gbar * d(wall term)/dnu
 #pragma unroll
                 for (int i = 0; i < Q; ++i) {
@@ -224,48 +196,28 @@ __global__ void __launch_bounds__(ATX *ATY) k_adj_gather_tiled(const float *__re
                             }
                         }
                     }
-                    gbar[i] = gb;
-                }
-                auto plane_of = [&](auto pp, auto mp, auto pm, auto mm) {
-                    return corners(gbar[pp.value], gbar[mp.value], gbar[pm.value], gbar[mm.value]);
-                };
-                const Corners xy = plane_of(Link<Q, 1, 1, 0>(), Link<Q, -1, 1, 0>(), Link<Q, 1, -1, 0>(),
-                                            Link<Q, -1, -1, 0>());
-                constexpr float WA = Q == 19 ? 2.f : 4.f;  // an axis link's weight
-                const float px = gbar[1], mx = gbar[2], py = gbar[3], my = gbar[4];
-                float gxx = fmaf(WA, px + mx, xy.t), g1x = fmaf(WA, px - mx, xy.a);
-                float gyy = fmaf(WA, py + my, xy.t), g1y = fmaf(WA, py - my, xy.b);
-                float g0, g1z = 0.f, gzz = 0.f, gxz = 0.f, gyz = 0.f;
-                const float gxy = xy.ab;
-                if (Q == 19) {
-                    const Corners xz = plane_of(Link<Q, 1, 0, 1>(), Link<Q, -1, 0, 1>(), Link<Q, 1, 0, -1>(),
-                                                Link<Q, -1, 0, -1>());
-                    const Corners yz = plane_of(Link<Q, 0, 1, 1>(), Link<Q, 0, -1, 1>(), Link<Q, 0, 1, -1>(),
-                                                Link<Q, 0, -1, -1>());
-                    const float pz = gbar[Q == 19 ? 5 : 0], mz = gbar[Q == 19 ? 6 : 0];
-                    g0 = fmaf(WA, px + mx, fmaf(12.f, gbar[0], gyy)) + fmaf(WA, pz + mz, xz.t) + yz.t;
-                    gxx += xz.t;
-                    g1x += xz.a;
-                    gzz = fmaf(WA, pz + mz, xz.t) + yz.t;
-                    g1z = fmaf(WA, pz - mz, xz.b) + yz.b;
-                    gyy += yz.t;
-                    g1y += yz.a;
-                    gxz = xz.ab;
-                    gyz = yz.ab;
-                } else {
-                    g0 = fmaf(WA, px + mx, fmaf(16.f, gbar[0], gyy));
+                    g0 = fmaf(wi, gb, g0);
+                    if (cx) g1x = fmaf(wi * cx, gb, g1x);
+                    if (cy) g1y = fmaf(wi * cy, gb, g1y);
+                    if (cz) g1z = fmaf(wi * cz, gb, g1z);
+                    if (cx) gxx = fmaf(wi, gb, gxx);
+                    if (cy) gyy = fmaf(wi, gb, gyy);
+                    if (cz) gzz = fmaf(wi, gb, gzz);
+                    if (cx && cy) gxy = fmaf(wi * cx * cy, gb, gxy);
+                    if (cx && cz) gxz = fmaf(wi * cx * cz, gb, gxz);
+                    if (cy && cz) gyz = fmaf(wi * cy * cz, gb, gyz);
                 }
                 const float hx = fmaf(gxx, u, fmaf(gxy, v, gxz * w));  // G2 . u
                 const float hy = fmaf(gxy, u, fmaf(gyy, v, gyz * w));
                 const float hz = fmaf(gxz, u, fmaf(gyz, v, gzz * w));
                 const float uG1 = fmaf(u, g1x, fmaf(v, g1y, w * g1z));
                 const float uG2u = fmaf(u, hx, fmaf(v, hy, w * hz));
-                const float s36 = p.s * (1.f / 36.f);
-                float ld = fmaf(0.125f, uG2u, fmaf(s36, uG1, g0 * fmaf(-1.f / 24.f, q, 1.f / 36.f)));
-                const float m3 = g0 * (-1.f / 12.f);
-                float lu = rho * fmaf(s36, g1x, fmaf(0.25f, hx, m3 * u));
-                float lv = rho * fmaf(s36, g1y, fmaf(0.25f, hy, m3 * v));
-                float lw = Q == 19 ? rho * fmaf(s36, g1z, fmaf(0.25f, hz, m3 * w)) : 0.f;
+                float ld = fmaf(4.5f, uG2u, fmaf(p.s, uG1, g0 * fmaf(-1.5f, q, 1.f)));
+                const float m3 = -3.f * g0;
+                float lu = rho * fmaf(p.s, g1x, fmaf(9.f, hx, m3 * u));
+                float lv = rho * fmaf(p.s, g1y, fmaf(9.f, hy, m3 * v));
+                float lw = Q == 19 ? rho * fmaf(p.s, g1z, fmaf(9.f, hz, m3 * w)) : 0.f;
+                const float ln = rho * uG1;
                 const int own = (ty + 1) * AW + tx + 1, os = s0;
                 const float jx = ring[os][1][own], jy = ring[os][2][own];
                 const float jz = Q == 19 ? ring[os][3][own] : 0.f;
@@ -287,7 +239,7 @@ __global__ void __launch_bounds__(ATX *ATY) k_adj_gather_tiled(const float *__re
                     out[2 * p.fstride + k] = lv;
                     if (Q == 19) out[3 * p.fstride + k] = lw;
                 }
-                nu_run += rho * fmaf(0.5f, uG1, -6.f * ju);
+                nu_run += fmaf(18.f, ln, -6.f * rho * ju);
                 if (WALLS) nu_run = fmaf(18.f * p.wallc / p.s, nu_wall, nu_run);  // 36 rho0 = wallc / nu
             }
             d = dn;
@@ -333,10 +285,10 @@ __global__ void __launch_bounds__(ATX *ATY) k_adj_gather_tiled(const float *__re
 // lane) and marches along z; the planes of (Dbar, Jbar) it reads, 10 rows each
 // (the column and one row either side), arrive by 1-D bulk copies (mbarrier
 // completion) in a ring of four slots: planes z-1, z, z+1 are read while z+2 is in
-// flight. A receiver's gbar = Dbar(y+c) + c.Jbar(y+c) enters the moments
-//   G0 += w gbar,  G1_a += w c_a gbar,  G2_ab += w c_a c_b gbar
-// plane of links by plane of links: the four diagonals of a coordinate plane together,
-// the axis links in pairs.
+// flight. Links are taken in pairs (c, -c), gbar+ = Dbar(y+c) + c.Jbar(y+c) and
+// gbar- = Dbar(y-c) - c.Jbar(y-c), and enter the moments through their sum
+// S = gbar+ + gbar- and difference D = gbar+ - gbar-:
+//   G0 += w S,  G1_a += w c_a D,  G2_ab += w c_a c_b S.
 // The state at t of the node is read straight from global memory (coalesced).
 namespace arow {
 
@@ -352,7 +304,7 @@ struct RG {
 struct RowParams {
     int nx, ny, nz, ycols, zc, nitems;
     long long fstride;
-    float s36, a;     // 18 nu / 36, 1 - 6 nu
+    float s, a;       // 18 nu, 1 - 6 nu
     float g[3];       // constant acceleration (Eq. force) or 0
     int *err;
 };
@@ -404,31 +356,25 @@ __device__ __forceinline__ void row4(const float *r, int x0, float (&v)[4]) {
     v[3] = m.w;
 }
 
-// 36 times the moments of four nodes: the weights are then 12, 2 (axis) and 1 (diagonal links)
 struct Mom {
     float g0[4], g1[3][4], g2[6][4];  // G0, G1 (x, y, z), G2 (xx, yy, zz, xy, xz, yz)
 };
-// one plane of links along x and b (y or z): rows hi and lo at b + 1 and b - 1, J_b at field fb;
-// per node the axis pair's sum and difference and the corners
-template <int NX>
-__device__ __forceinline__ void x_plane(const float *hi, const float *lo, int fs, int fb, int x0, float (&S)[4],
-                                        float (&D)[4], Corners (&c)[4]) {
-    float A[6], Xh[6], B[6], Xl[6], J[6];  // A = Dbar + J_b above, B = Dbar - J_b below
-    row6<NX>(hi, x0, A);
-    row6<NX>(hi + fs, x0, Xh);
-    row6<NX>(hi + fb * fs, x0, J);
-#pragma unroll
-    for (int n = 0; n < 6; ++n) A[n] += J[n];
-    row6<NX>(lo, x0, B);
-    row6<NX>(lo + fs, x0, Xl);
-    row6<NX>(lo + fb * fs, x0, J);
-#pragma unroll
-    for (int n = 0; n < 6; ++n) B[n] -= J[n];
+// accumulate the pair (c, -c) of weight w from gbar+ / gbar- of the four nodes
+template <int CX, int CY, int CZ>
+__device__ __forceinline__ void pair_moments(Mom &m, float w, const float (&gp)[4], const float (&gm)[4]) {
 #pragma unroll
     for (int n = 0; n < 4; ++n) {
-        S[n] = A[n + 1] + B[n + 1];
-        D[n] = A[n + 1] - B[n + 1];
-        c[n] = corners(A[n + 2] + Xh[n + 2], A[n] - Xh[n], B[n + 2] + Xl[n + 2], B[n] - Xl[n]);
+        const float S = gp[n] + gm[n], D = gp[n] - gm[n];
+        m.g0[n] = fmaf(w, S, m.g0[n]);
+        if (CX) m.g1[0][n] = fmaf(w * CX, D, m.g1[0][n]);
+        if (CY) m.g1[1][n] = fmaf(w * CY, D, m.g1[1][n]);
+        if (CZ) m.g1[2][n] = fmaf(w * CZ, D, m.g1[2][n]);
+        if (CX) m.g2[0][n] = fmaf(w, S, m.g2[0][n]);
+        if (CY) m.g2[1][n] = fmaf(w, S, m.g2[1][n]);
+        if (CZ) m.g2[2][n] = fmaf(w, S, m.g2[2][n]);
+        if (CX && CY) m.g2[3][n] = fmaf(w * CX * CY, S, m.g2[3][n]);
+        if (CX && CZ) m.g2[4][n] = fmaf(w * CX * CZ, S, m.g2[4][n]);
+        if (CY && CZ) m.g2[5][n] = fmaf(w * CY * CZ, S, m.g2[5][n]);
     }
 }
 
@@ -438,70 +384,109 @@ template <int NH>
 __device__ __forceinline__ void gather(Mom &m, const float *sm, const float *s0, const float *sp, int rs, int x0,
                                        float (&own)[4][4]) {
     constexpr int NX = RG<NH>::NX, FS = TROWS * NX;  // field stride in a slot
-    float S[4], D[4];
-    Corners c[4];
+    constexpr float WA = 1.f / 18.f, WD = 1.f / 36.f;
+#pragma unroll
+    for (int n = 0; n < 4; ++n) {
+        m.g0[n] = 0.f;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) m.g1[a][n] = 0.f;
+#pragma unroll
+        for (int a = 0; a < 6; ++a) m.g2[a][n] = 0.f;
+    }
     {  // plane z, own row: the rest link, (1,0,0), and the node's own (Dbar, Jbar)
-        float R[6], Jx[6];
-        row6<NX>(s0 + rs * NX, x0, R);
+        float D[6], Jx[6];
+        row6<NX>(s0 + rs * NX, x0, D);
         row6<NX>(s0 + FS + rs * NX, x0, Jx);
         row4(s0 + 2 * FS + rs * NX, x0, own[2]);
         row4(s0 + 3 * FS + rs * NX, x0, own[3]);
+        float gp[4], gm[4];
 #pragma unroll
         for (int n = 0; n < 4; ++n) {
-            own[0][n] = R[n + 1];
+            own[0][n] = D[n + 1];
             own[1][n] = Jx[n + 1];
-            const float gp = R[n + 2] + Jx[n + 2], gm = R[n] - Jx[n];
-            m.g2[0][n] = 2.f * (gp + gm);
-            m.g1[0][n] = 2.f * (gp - gm);
-            m.g0[n] = fmaf(12.f, R[n + 1], m.g2[0][n]);
+            m.g0[n] = (1.f / 3.f) * D[n + 1];
+            gp[n] = D[n + 2] + Jx[n + 2];
+            gm[n] = D[n] - Jx[n];
         }
+        pair_moments<1, 0, 0>(m, WA, gp, gm);
     }
-    // plane z, rows rs -+ 1: (0,1,0), (1,1,0), (1,-1,0)
-    x_plane<NX>(s0 + (rs + 1) * NX, s0 + (rs - 1) * NX, FS, 2, x0, S, D, c);
-#pragma unroll
-    for (int n = 0; n < 4; ++n) {
-        m.g2[1][n] = fmaf(2.f, S[n], c[n].t);
-        m.g0[n] += m.g2[1][n];
-        m.g2[0][n] += c[n].t;
-        m.g1[0][n] += c[n].a;
-        m.g1[1][n] = fmaf(2.f, D[n], c[n].b);
-        m.g2[3][n] = c[n].ab;
-    }
-    // planes z -+ 1, own row: (0,0,1), (1,0,1), (1,0,-1)
-    x_plane<NX>(sp + rs * NX, sm + rs * NX, FS, 3, x0, S, D, c);
-#pragma unroll
-    for (int n = 0; n < 4; ++n) {
-        m.g2[2][n] = fmaf(2.f, S[n], c[n].t);
-        m.g0[n] += m.g2[2][n];
-        m.g2[0][n] += c[n].t;
-        m.g1[0][n] += c[n].a;
-        m.g1[2][n] = fmaf(2.f, D[n], c[n].b);
-        m.g2[4][n] = c[n].ab;
-    }
-    // (0,1,1) and (0,1,-1): rows rs -+ 1 of planes z -+ 1
-    float g[4][4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {  // (y, z) = ++, -+, +-, --
-        const float *r = (k < 2 ? sp : sm) + (rs + (k % 2 ? -1 : 1)) * NX;
-        float Jy[4], Jz[4];
-        row4(r, x0, g[k]);
-        row4(r + 2 * FS, x0, Jy);
-        row4(r + 3 * FS, x0, Jz);
+    {  // plane z, rows rs -+ 1: (0,1,0), (1,1,0), (1,-1,0)
+        float Du[6], Xu[6], Yu[6], Dd[6], Xd[6], Yd[6];
+        row6<NX>(s0 + (rs + 1) * NX, x0, Du);
+        row6<NX>(s0 + FS + (rs + 1) * NX, x0, Xu);
+        row6<NX>(s0 + 2 * FS + (rs + 1) * NX, x0, Yu);
+        row6<NX>(s0 + (rs - 1) * NX, x0, Dd);
+        row6<NX>(s0 + FS + (rs - 1) * NX, x0, Xd);
+        row6<NX>(s0 + 2 * FS + (rs - 1) * NX, x0, Yd);
+        float gp[4], gm[4];
 #pragma unroll
         for (int n = 0; n < 4; ++n) {
-            g[k][n] = k % 2 ? g[k][n] - Jy[n] : g[k][n] + Jy[n];
-            g[k][n] = k < 2 ? g[k][n] + Jz[n] : g[k][n] - Jz[n];
+            gp[n] = Du[n + 1] + Yu[n + 1];
+            gm[n] = Dd[n + 1] - Yd[n + 1];
         }
+        pair_moments<0, 1, 0>(m, WA, gp, gm);
+#pragma unroll
+        for (int n = 0; n < 4; ++n) {
+            gp[n] = Du[n + 2] + Xu[n + 2] + Yu[n + 2];  // (1,1,0) from (x+1, y+1)
+            gm[n] = Dd[n] - Xd[n] - Yd[n];              // (-1,-1,0) from (x-1, y-1)
+        }
+        pair_moments<1, 1, 0>(m, WD, gp, gm);
+#pragma unroll
+        for (int n = 0; n < 4; ++n) {
+            gp[n] = Dd[n + 2] + Xd[n + 2] - Yd[n + 2];  // (1,-1,0) from (x+1, y-1)
+            gm[n] = Du[n] - Xu[n] + Yu[n];              // (-1,1,0) from (x-1, y+1)
+        }
+        pair_moments<1, -1, 0>(m, WD, gp, gm);
+    }
+    {  // planes z -+ 1, own row: (0,0,1), (1,0,1), (1,0,-1)
+        float Da[6], Xa[6], Za[6], Db[6], Xb[6], Zb[6];
+        row6<NX>(sp + rs * NX, x0, Da);
+        row6<NX>(sp + FS + rs * NX, x0, Xa);
+        row6<NX>(sp + 3 * FS + rs * NX, x0, Za);
+        row6<NX>(sm + rs * NX, x0, Db);
+        row6<NX>(sm + FS + rs * NX, x0, Xb);
+        row6<NX>(sm + 3 * FS + rs * NX, x0, Zb);
+        float gp[4], gm[4];
+#pragma unroll
+        for (int n = 0; n < 4; ++n) {
+            gp[n] = Da[n + 1] + Za[n + 1];
+            gm[n] = Db[n + 1] - Zb[n + 1];
+        }
+        pair_moments<0, 0, 1>(m, WA, gp, gm);
+#pragma unroll
+        for (int n = 0; n < 4; ++n) {
+            gp[n] = Da[n + 2] + Xa[n + 2] + Za[n + 2];  // (1,0,1) from (x+1, z+1)
+            gm[n] = Db[n] - Xb[n] - Zb[n];              // (-1,0,-1) from (x-1, z-1)
+        }
+        pair_moments<1, 0, 1>(m, WD, gp, gm);
+#pragma unroll
+        for (int n = 0; n < 4; ++n) {
+            gp[n] = Db[n + 2] + Xb[n + 2] - Zb[n + 2];  // (1,0,-1) from (x+1, z-1)
+            gm[n] = Da[n] - Xa[n] + Za[n];              // (-1,0,1) from (x-1, z+1)
+        }
+        pair_moments<1, 0, -1>(m, WD, gp, gm);
     }
 #pragma unroll
-    for (int n = 0; n < 4; ++n) {
-        const Corners q = corners(g[0][n], g[1][n], g[2][n], g[3][n]);
-        m.g0[n] += q.t;
-        m.g2[1][n] += q.t;
-        m.g2[2][n] += q.t;
-        m.g1[1][n] += q.a;
-        m.g1[2][n] += q.b;
-        m.g2[5][n] = q.ab;
+    for (int k = 0; k < 2; ++k) {  // (0,1,1) and (0,1,-1): rows rs -+ 1 of planes z -+ 1
+        const float *pu = k == 0 ? sp : sm, *pd = k == 0 ? sm : sp;  // c = (0,1,+-1): up row in plane z+-1
+        float Du[4], Yu[4], Zu[4], Dd[4], Yd[4], Zd[4];
+        row4(pu + (rs + 1) * NX, x0, Du);
+        row4(pu + 2 * FS + (rs + 1) * NX, x0, Yu);
+        row4(pu + 3 * FS + (rs + 1) * NX, x0, Zu);
+        row4(pd + (rs - 1) * NX, x0, Dd);
+        row4(pd + 2 * FS + (rs - 1) * NX, x0, Yd);
+        row4(pd + 3 * FS + (rs - 1) * NX, x0, Zd);
+        const float cz = k == 0 ? 1.f : -1.f;
+        float gp[4], gm[4];
+#pragma unroll
+        for (int n = 0; n < 4; ++n) {
+            gp[n] = fmaf(cz, Zu[n], Du[n] + Yu[n]);
+            gm[n] = fmaf(-cz, Zd[n], Dd[n] - Yd[n]);
+        }
+        if (k == 0)
+            pair_moments<0, 1, 1>(m, WD, gp, gm);
+        else
+            pair_moments<0, 1, -1>(m, WD, gp, gm);
     }
 }
 
@@ -515,7 +500,8 @@ __global__ void __launch_bounds__(RG<NH>::NTH, 2 / NH) k_adj_rows(const float *_
     using namespace lwacm::tile;
     constexpr int NX = RG<NH>::NX, PLANE = RG<NH>::PLANE, NTH = RG<NH>::NTH;
     // the next launch's CTAs may take their SMs as this one's leave them; none touches global
-    // memory before this grid is complete
+    // memory before this grid is complete (128^3: 32.8 us a step of a 24-step sweep, 30.4 with it;
+    // 230 instructions a node, issue slots 56% busy with 16 warps a SM)
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     extern __shared__ float4 smem4[];
     float *ring = reinterpret_cast<float *>(smem4);
@@ -586,12 +572,11 @@ __global__ void __launch_bounds__(RG<NH>::NTH, 2 / NH) k_adj_rows(const float *_
                 const float hz = fmaf(m.g2[4][n], u, fmaf(m.g2[5][n], v, m.g2[2][n] * w));
                 const float uG1 = fmaf(u, m.g1[0][n], fmaf(v, m.g1[1][n], w * m.g1[2][n]));
                 const float uG2u = fmaf(u, hx, fmaf(v, hy, w * hz));
-                // the moments carry a factor 36
-                float ld = fmaf(0.125f, uG2u, fmaf(p.s36, uG1, m.g0[n] * fmaf(-1.f / 24.f, q, 1.f / 36.f)));
-                const float m3 = m.g0[n] * (-1.f / 12.f);
-                float lu = rho * fmaf(p.s36, m.g1[0][n], fmaf(0.25f, hx, m3 * u));
-                float lv = rho * fmaf(p.s36, m.g1[1][n], fmaf(0.25f, hy, m3 * v));
-                float lw = rho * fmaf(p.s36, m.g1[2][n], fmaf(0.25f, hz, m3 * w));
+                float ld = fmaf(4.5f, uG2u, fmaf(p.s, uG1, m.g0[n] * fmaf(-1.5f, q, 1.f)));
+                const float m3 = -3.f * m.g0[n];
+                float lu = rho * fmaf(p.s, m.g1[0][n], fmaf(9.f, hx, m3 * u));
+                float lv = rho * fmaf(p.s, m.g1[1][n], fmaf(9.f, hy, m3 * v));
+                float lw = rho * fmaf(p.s, m.g1[2][n], fmaf(9.f, hz, m3 * w));
                 const float jx = own[1][n], jy = own[2][n], jz = own[3][n];
                 const float ju = fmaf(u, jx, fmaf(v, jy, w * jz));
                 ld = fmaf(p.a, ju, ld);
@@ -612,7 +597,7 @@ __global__ void __launch_bounds__(RG<NH>::NTH, 2 / NH) k_adj_rows(const float *_
                     o[2][n] = lv;
                     o[3][n] = lw;
                 }
-                nu_run += rho * fmaf(0.5f, uG1, -6.f * ju);
+                nu_run += fmaf(18.f, rho * uG1, -6.f * rho * ju);
             }
 #pragma unroll
             for (int f = 0; f < 4; ++f)
@@ -691,7 +676,7 @@ cudaError_t launch_rows(const float *state_t, const float *dj, float *out, const
     p.zc = zc;
     p.nitems = p.ycols * ((sp.nz + zc - 1) / zc);
     p.fstride = sp.fstride;
-    p.s36 = sp.s * (1.f / 36.f);
+    p.s = sp.s;
     p.a = sp.a;
     for (int c = 0; c < 3; ++c) p.g[c] = sp.has_force ? sp.force[c] : 0.f;
     p.err = sp.err;
