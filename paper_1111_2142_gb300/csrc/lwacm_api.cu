@@ -43,6 +43,7 @@ struct lwacm_ctx {
     bool sr = false;          // BF16 / FP16 stores rounded stochastically (half-row kernel)
     bool no_cluster = false;  // the device does not take the cluster kernel
     bool march = false;       // kernel 5, automatic choice: by warps that march along z (kernels_rows3.cu)
+    bool recording = false;   // the steps of a recorded run (step_between)
     bool scalar_rows = false; // the passive scalar on its own kernel after the half-row flow kernel
     bool scalar_march = false;  // on its own marching kernel after the general flow kernel
     int nsc = 0;              // fields stored after the flow fields: the scalar or the trace (0 or 1)
@@ -334,7 +335,14 @@ cudaError_t step_between(lwacm_ctx *c, const void *in, void *out, cudaStream_t s
     cudaError_t e = cudaSuccess;
     if (c->kernel == 5 && p.sdelta != 0.f) e = launch_nup_sum(c->storage, in, p.nup_p, p, st);
     if (e != cudaSuccess) return e;
-    e = c->march                     ? launch_step_rows3d(c->storage, in, out, p, st)
+    // Recorded runs and their recomputation stay on the half-row, 2D-tile and gather kernels: dL/dnu
+    // is a sum that may cancel, and the marching kernels' other order of additions moved it by more
+    // than 2e-5 in one of five random runs
+    const bool rec = c->recording;
+    e = rec && c->kernel == 6        ? launch_step_tiles2d(c->Q, c->storage, c->batch_shape > 0 ? c->batch_shape : 2, in,
+                                                           out, p, st)
+                    : rec && c->kernel == 1 ? launch_step_gather(c->Q, c->storage, in, out, p, st)
+                    : c->march && !rec ? launch_step_rows3d(c->storage, in, out, p, st)
                     : c->kernel == 5 ? launch_step_half(c->Q, c->storage, in, out, pf, st)
                     : c->kernel == 6 && c->batch_shape == 0 ? launch_step_rows2d(c->storage, in, out, p, st)
                     : c->kernel == 6 ? launch_step_tiles2d(c->Q, c->storage, c->batch_shape, in, out, p, st)
@@ -342,10 +350,11 @@ cudaError_t step_between(lwacm_ctx *c, const void *in, void *out, cudaStream_t s
     if (e != cudaSuccess) return e;
     // the D2Q9 and the marching D3Q19 kernels apply the wall rule themselves; the half-row
     // kernel the x-face walls of a cavity whose lid is not on an x face
-    const bool walls_done = c->kernel == 6 || ((c->march || c->kernel == 1) && c->Q == 19 && rows3d_walls(p));
+    const bool walls_done =
+        c->kernel == 6 || (!rec && (c->march || c->kernel == 1) && c->Q == 19 && rows3d_walls(p));
     if (c->bc != LWACM_BC_PERIODIC && !walls_done) {
         StepParams pw = p;
-        pw.xfaces_done = c->kernel == 5 && !c->march && half_xwalls(p) ? 1 : 0;
+        pw.xfaces_done = c->kernel == 5 && (rec || !c->march) && half_xwalls(p) ? 1 : 0;
         e = launch_wall_pass(c->Q, c->storage, in, out, pw, st);
     }
     if (e == cudaSuccess && p.sr_ctr && c->kernel == 5) e = launch_sr_tick(p.sr_ctr, st);
@@ -366,8 +375,23 @@ cudaError_t enqueue_step(lwacm_ctx *c, int cur, cudaStream_t st) {
 // kernel. A launch costs 8 us, single steps 2.1 to 2.5 each where no graph is replayed (64^2: 4
 // steps 10.9 us against 15.7, 2 steps 12.0 against 13.7).
 bool on_cluster(const lwacm_ctx *c, long long n) {
-    return n >= 4 && c->kernel == 6 && c->batch_shape == 0 && !c->semi && !c->no_cluster && cluster2d_supported(params(c));
+    return n >= 4 && !c->recording && c->kernel == 6 && c->batch_shape == 0 && !c->semi && !c->no_cluster && cluster2d_supported(params(c));
 }
+
+// the steps of a recorded run, while it lives; graphs of other steps are not replayed in it nor its own
+// after it (runs whose segments are shorter than a graph capture none)
+struct Recording {
+    lwacm_ctx *c;
+    bool graphs;
+    Recording(lwacm_ctx *c_, long long seg) : c(c_), graphs(c_->graph_chunk > 0 && seg >= c_->graph_chunk) {
+        c->recording = true;
+        if (graphs) drop_graphs(c);
+    }
+    ~Recording() {
+        c->recording = false;
+        if (graphs) drop_graphs(c);
+    }
+};
 
 // adjoint workspace: K checkpoints, S+1 segment states, 2 lambda / (Dbar, Jbar)
 // states, one more (Dbar, Jbar) state, dL/dnu partials, total and block counter
@@ -1123,6 +1147,7 @@ lwacm_status lwacm_forward_record(lwacm_ctx *c, long long T, int stride, void *w
     c->adj_bytes = bytes;
     const size_t sb = (size_t)c->Nal * 4 * c->nf;
     c->rec_last_kept = false;
+    const Recording rec(c, L.S);
     for (long long k = 0; k < L.K; ++k) {
         char *ck = c->adj + L.ckpt + k * L.state;
         CK(c, cudaMemcpyAsync(ck, bufp(c, c->cur), sb, cudaMemcpyDeviceToDevice, c->stream), "checkpoint copy");
@@ -1172,6 +1197,7 @@ lwacm_status lwacm_backward(lwacm_ctx *c, const void *ld, const void *lux, const
     CK(c, launch_convert_in_fields(STORE_F32, dtype, lin, c->nf, lam0, c->Nal, c->N, c->stream), "lambda in");
     CK(c, cudaMemsetAsync(total, 0, 16, c->stream), "clear dnu");
     const StepParams p = params(c);
+    const Recording rec(c, 0);  // recomputed segments; no graph
     int cur = 0;
     for (long long k = L.K - 1; k >= 0; --k) {
         const long long t0 = k * L.S;
