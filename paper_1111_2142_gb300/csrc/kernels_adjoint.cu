@@ -491,17 +491,16 @@ __device__ __forceinline__ void gather(Mom &m, const float *sm, const float *s0,
 }
 
 template <int NH, bool NEXT>
-__global__ void __launch_bounds__(RG<NH>::NTH, 2 / NH) k_adj_rows(const float *__restrict__ st,
-                                                                 const float *__restrict__ dj,
-                                                                 float *__restrict__ out, RowParams p,
-                                                                 double *__restrict__ nu_partial,
-                                                                 unsigned *__restrict__ done,
-                                                                 double *__restrict__ nu_total) {
+__global__ void __launch_bounds__(RG<NH>::NTH, 2 / NH) k_adj_rows(const float *st, const float *dj, float *out,
+                                                                 RowParams p, double *nu_partial, unsigned *done,
+                                                                 double *nu_total) {
     using namespace lwacm::tile;
     constexpr int NX = RG<NH>::NX, PLANE = RG<NH>::PLANE, NTH = RG<NH>::NTH;
     // the next launch's CTAs may take their SMs as this one's leave them; none touches global
     // memory before this grid is complete (128^3: 32.8 us a step of a 24-step sweep, 30.4 with it;
-    // 230 instructions a node, issue slots 56% busy with 16 warps a SM)
+    // 230 instructions a node, issue slots 56% busy with 16 warps a SM). The grid before may
+    // write what this one reads until then, so no pointer is marked const __restrict__: such
+    // loads may take the read-only path, which griddepcontrol.wait does not order
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     extern __shared__ float4 smem4[];
     float *ring = reinterpret_cast<float *>(smem4);

@@ -319,8 +319,7 @@ __device__ __forceinline__ void rows2_update(const T *in, T *out, const BatchRow
 // (fewer CTAs to start).
 constexpr int rows_warps(int ns) { return ns == 1 ? 4 : 1; }
 template <int NS, typename T>
-__global__ void __launch_bounds__(32 * rows_warps(NS)) k_batch_rows(const T *__restrict__ in, T *__restrict__ out,
-                                                                    BatchParams bp) {
+__global__ void __launch_bounds__(32 * rows_warps(NS)) k_batch_rows(const T *in, T *out, BatchParams bp) {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const long long t = rows_warps(NS) == 1 ? (long long)blockIdx.x
                                             : (long long)blockIdx.x * rows_warps(NS) + (threadIdx.x >> 5);

@@ -39,7 +39,7 @@ using namespace rows2;
 // numbered along x first, so that neighbours read the same rows at the same time.
 template <int NS, typename T, bool WALLS, bool FIELD, bool BULK, bool NUP>
 __global__ void __launch_bounds__(32 * (NS == 1 ? kMaxWarps : 1))
-    k_d2q9_rows(const T *__restrict__ in, T *__restrict__ out, Dom2 dm, int ctasx, int rows, Walls2 wl, Force2 fc,
+    k_d2q9_rows(const T *in, T *out, Dom2 dm, int ctasx, int rows, Walls2 wl, Force2 fc,
                 float gamma, float sdelta) {
     // the next step's CTAs may take their SMs as this step's leave them; none touches
     // global memory before this grid is complete

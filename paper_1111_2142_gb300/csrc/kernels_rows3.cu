@@ -114,15 +114,17 @@ struct March3 {
     struct Raw {
         T f[4][6];
     };
+    // ordinary loads: the grid before may still write what this one reads until
+    // griddepcontrol.wait (ldraw, rows2.cuh)
     __device__ __forceinline__ void load(int z, Raw &r) const {
         z = z < 0 ? z + dm.nz : (z >= dm.nz ? z - dm.nz : z);
 #pragma unroll
         for (int f = 0; f < 4; ++f) {
             const T *p = in + (z * plane + f * dm.fstride);
-            r.f[f][0] = __ldg(byte_at(p, lo));
+            r.f[f][0] = *byte_at(p, lo);
 #pragma unroll
-            for (int j = 0; j < kTile; ++j) r.f[f][1 + j] = __ldg(byte_at(p + (long long)j * dm.nx, off));
-            r.f[f][5] = __ldg(byte_at(p, hi));
+            for (int j = 0; j < kTile; ++j) r.f[f][1 + j] = *byte_at(p + (long long)j * dm.nx, off);
+            r.f[f][5] = *byte_at(p, hi);
         }
     }
 
@@ -388,8 +390,8 @@ struct March3 {
             for (int c = 0; c < 3; ++c) {
                 const float *q = dm.field + (z * plane + c * dm.fstride);
                 const long long nx = dm.nx;
-                g[0][c] = make_float2(__ldg(byte_at(q, off * K)), __ldg(byte_at(q + 2 * nx, off * K)));
-                g[1][c] = make_float2(__ldg(byte_at(q + nx, off * K)), __ldg(byte_at(q + 3 * nx, off * K)));
+                g[0][c] = make_float2(*byte_at(q, off * K), *byte_at(q + 2 * nx, off * K));
+                g[1][c] = make_float2(*byte_at(q + nx, off * K), *byte_at(q + 3 * nx, off * K));
             }
         }
         Sum3 N[2];
@@ -455,8 +457,7 @@ struct March3 {
 // the neighbours of a strip pass each plane together and share its lines in L2 (runs of
 // equal length that cross from column to column, out of step, took 235 us on 256^3)
 template <typename T, bool FIELD, bool WALLS>
-__global__ void __launch_bounds__(32 * kWarps) k_d3q19_rows(const T *__restrict__ in, T *__restrict__ out, Dom3 dm,
-                                                            int strips, int groups, int runs) {
+__global__ void __launch_bounds__(32 * kWarps) k_d3q19_rows(const T *in, T *out, Dom3 dm, int strips, int groups, int runs) {
     // the next step's CTAs may take their SMs as this step's leave them; none touches
     // global memory before this grid is complete
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

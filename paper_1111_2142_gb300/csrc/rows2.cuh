@@ -133,10 +133,14 @@ template <typename T>
 __device__ __forceinline__ const T *byte_at(const T *p, unsigned bytes) {
     return (const T *)((const char *)p + bytes);
 }
-// stored elements as loaded: widened when used, so that a load in flight holds nothing up
+// stored elements as loaded: widened when used, so that a load in flight holds nothing up.
+// Ordinary loads and not __ldg: a grid launched with programmatic stream serialization is
+// alive while the grid before it still writes what this one reads, and the read-only path is
+// defined only for data that nobody writes during the kernel (griddepcontrol.wait orders
+// ordinary loads). COHERENT: past L1, for what other CTAs of the same launch write.
 template <bool COHERENT, typename T>
 __device__ __forceinline__ T ldraw(const T *p) {
-    return COHERENT ? __ldcg(p) : __ldg(p);
+    return COHERENT ? __ldcg(p) : *p;
 }
 __device__ __forceinline__ float widen(float v) { return v; }
 __device__ __forceinline__ float widen(__nv_bfloat16 v) { return __bfloat162float(v); }
@@ -247,7 +251,7 @@ struct March {
 #pragma unroll
             for (int f = 0; f < 2; ++f)
 #pragma unroll
-                for (int h = 0; h < NS; ++h) r.g[f][h] = __ldg(fc.field + (row + f * dm.fstride) + xo[h]);
+                for (int h = 0; h < NS; ++h) r.g[f][h] = fc.field[(row + f * dm.fstride) + xo[h]];
     }
     static __device__ __forceinline__ float pick(const T (&v)[1]) { return widen(v[0]); }
     static __device__ __forceinline__ F2 pick(const T (&v)[2]) { return make_float2(widen(v[0]), widen(v[1])); }
