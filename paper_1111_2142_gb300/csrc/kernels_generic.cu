@@ -855,6 +855,20 @@ static cudaError_t from_t(int src_dtype, const Sources &src, int nf, void *dst, 
 
 cudaError_t launch_convert_in_fields(int storage, int src_dtype, const void *const *src, int nf, void *dst,
                                      long long stride, long long n, cudaStream_t st) {
+    // A source may lie in the destination (the state handed back through its own views): where one
+    // array is read from what another one is copied to, in turn, array f after those before it
+    const long long sb = src_dtype == XFER_F64 ? 8 : 4, db = storage == STORE_F32 ? 4 : 2;
+    for (int f = 0; f < nf; ++f)
+        for (int g = 0; g < nf; ++g) {
+            const char *a = (const char *)src[f], *b = (const char *)dst + g * stride * db;
+            if (f == g || a + n * sb <= b || b + n * db <= a) continue;
+            for (int k = 0; k < nf; ++k) {
+                const cudaError_t e =
+                    launch_convert_in(storage, src_dtype, src[k], (char *)dst + k * stride * db, n, st);
+                if (e != cudaSuccess) return e;
+            }
+            return cudaSuccess;
+        }
     Sources s = {};
     for (int f = 0; f < nf; ++f) s.p[f] = src[f];
     switch (storage) {

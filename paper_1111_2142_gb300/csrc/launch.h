@@ -27,7 +27,8 @@ cudaError_t launch_semi_implicit(int Q, int storage, const void *in, void *out, 
                                  cudaStream_t st);
 cudaError_t launch_convert_in(int storage, int src_dtype, const void *src, void *dst, long long n,
                               cudaStream_t st);
-// nf (at most four) arrays on the device, array f to dst + f stride
+// nf (at most four) arrays on the device, array f to dst + f stride; one after the other where
+// a source overlaps the destination of another array
 cudaError_t launch_convert_in_fields(int storage, int src_dtype, const void *const *src, int nf, void *dst,
                                      long long stride, long long n, cudaStream_t st);
 cudaError_t launch_convert_out(int storage, int dst_dtype, const void *src, void *dst, long long n,

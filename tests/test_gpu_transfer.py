@@ -36,6 +36,26 @@ def test_fields_from_device_arrays(lw, shape, storage, dtype, shift):
     sim.close()
 
 
+@pytest.mark.parametrize("shape", [(1, 1, 3), (5, 6, 7), (24, 80, 100)])
+@pytest.mark.parametrize("order", [(0, 2, 3, None), (1, 2, 3, None), (0, 2, 1, 3), (3, 3, 0, 1), (0, 1, 2, 3)])
+def test_fields_from_views_of_the_state(shape, order, lw):
+    """The state's own views as sources: the arrays are copied one after the other, so that field k
+    takes what its source holds once the fields before it are in place (None: another array)."""
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(83)
+    f = [torch.randn(shape, generator=g, device="cuda") * 0.05 for _ in range(5)]
+    sim = lw.Lwacm(19, shape[2], shape[1], shape[0], 0.02)
+    sim.set_fields(*f[:4])
+    views = list(sim.fields())
+    want = [t.clone() for t in f[:4]]
+    for k, o in enumerate(order):
+        want[k] = f[4].clone() if o is None else want[o].clone()
+    sim.set_fields(*[f[4] if o is None else views[o] for o in order])
+    for a, v in zip(want, sim.fields()):
+        assert torch.equal(a, v)
+    sim.close()
+
+
 @pytest.mark.parametrize("dtype", ["float32", "float64"])
 def test_force_field_from_unaligned_arrays(lw, dtype):
     """A force field from arrays one element past a 16-byte boundary acts as from aligned ones."""
