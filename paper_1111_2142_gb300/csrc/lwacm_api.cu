@@ -393,6 +393,17 @@ struct Recording {
     }
 };
 
+// whether n arrays lie in the current GPU's own memory
+bool all_local(const void *const *p, int n) {
+    int dev = 0;
+    bool ok = cudaGetDevice(&dev) == cudaSuccess;
+    for (int k = 0; k < n && ok; ++k) {
+        cudaPointerAttributes a;
+        ok = cudaPointerGetAttributes(&a, p[k]) == cudaSuccess && a.type == cudaMemoryTypeDevice && a.device == dev;
+    }
+    return ok;
+}
+
 // adjoint workspace: K checkpoints, S+1 segment states, 2 lambda / (Dbar, Jbar)
 // states, one more (Dbar, Jbar) state, dL/dnu partials, total and block counter
 struct AdjLayout {
@@ -898,13 +909,17 @@ lwacm_status lwacm_set_force_field(lwacm_ctx *c, const void *gx, const void *gy,
     const void *src[3] = {gx, gy, gz};
     const size_t sb = dtype == LWACM_F64 ? 8 : 4;
     const size_t nbytes = (size_t)c->N * sb;
-    if (where == LWACM_DEVICE)
+    // device arrays by one launch; FP32 ones that are not this GPU's (another GPU's, which a kernel
+    // may have no access to) by copies
+    const bool one = where == LWACM_DEVICE && (dtype == LWACM_F64 || all_local(src, c->D));
+    if (one)
         CK(c, launch_convert_in_fields(STORE_F32, dtype, src, c->D, c->ws + c->off_ff, c->Nal, c->N, c->stream),
            "force field copy");
-    for (int a = 0; a < c->D && where == LWACM_HOST; ++a) {
+    for (int a = 0; a < c->D && !one; ++a) {
         char *dst = c->ws + c->off_ff + (size_t)a * c->Nal * 4;
         if (dtype == LWACM_F32) {
-            CK(c, cudaMemcpyAsync(dst, src[a], nbytes, cudaMemcpyHostToDevice, c->stream), "force field copy");
+            const cudaMemcpyKind kind = where == LWACM_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDefault;
+            CK(c, cudaMemcpyAsync(dst, src[a], nbytes, kind, c->stream), "force field copy");
             continue;
         }
         CK(c, cudaMemcpyAsync(c->ws + c->off_stage, src[a], nbytes, cudaMemcpyHostToDevice, c->stream), "H2D stage");

@@ -1,5 +1,7 @@
 """Fields and forces copied in by one launch for all arrays: vector and single loads (aligned
 and unaligned sources, counts that are no multiple of four), every type."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -73,3 +75,45 @@ def test_force_field_from_unaligned_arrays(lw, dtype):
     for x, y in zip(*out):
         assert np.array_equal(x, y)
     assert float(np.max(np.abs(out[0][1]))) > 1e-5
+
+
+def test_force_field_from_memory_of_another_device(lw):
+    """An FP32 force array that is not in this GPU's memory goes through a copy and not through a
+    kernel that reads it, which may have no access to it. Pinned host memory stands in for another
+    GPU's; the nodes of a captured call show the route."""
+    import torch
+    n = 24 * 20
+    sim = lw.Lwacm(9, 24, 20, 1, 0.02, force_field=True, stream=torch.cuda.Stream())
+    sim.set_fields(*[np.zeros((20, 24))] * 3)
+    host = [(torch.arange(n, dtype=torch.float32) * s).pin_memory() for s in (1e-6, -2e-6)]
+    here = [t.cuda() for t in host]
+    torch.cuda.synchronize()
+
+    def nodes(arrays):
+        sim.set_force_field(*here)  # on already: nothing is chosen anew under capture
+        sim.sync()
+        g = torch.cuda.CUDAGraph(keep_graph=True)
+        with torch.cuda.graph(g, stream=sim.stream):
+            status = sim._lib.lwacm_set_force_field(sim._h, *[t.data_ptr() for t in arrays], None, lw.F32, lw.DEVICE)
+        assert status == lw.OK
+        cu, graph, count = ctypes.CDLL("libcuda.so.1"), ctypes.c_void_p(g.raw_cuda_graph()), ctypes.c_size_t()
+        assert cu.cuGraphGetNodes(graph, None, ctypes.byref(count)) == 0
+        found, kind, kinds = (ctypes.c_void_p * count.value)(), ctypes.c_int(), []
+        assert cu.cuGraphGetNodes(graph, found, ctypes.byref(count)) == 0
+        for node in found:
+            assert cu.cuGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)) == 0
+            kinds.append(kind.value)
+        return kinds
+
+    assert nodes(here) == [0]  # one kernel
+    assert nodes(host) == [1, 1]  # two copies
+    out = []
+    for arrays in (here, host):
+        sim.set_fields(*[np.zeros((20, 24))] * 3)
+        assert sim._lib.lwacm_set_force_field(sim._h, *[t.data_ptr() for t in arrays], None, lw.F32, lw.DEVICE) == lw.OK
+        sim.step(3)
+        out.append(sim.get_fields())
+    for x, y in zip(*out):
+        assert np.array_equal(x, y)
+    assert float(np.max(np.abs(out[0][1]))) > 1e-5
+    sim.close()
