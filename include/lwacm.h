@@ -385,7 +385,22 @@ const char *lwacm_last_error(const lwacm_ctx *ctx);
 lwacm_status lwacm_autotune(lwacm_ctx *ctx, const char *cache_path, int trial_steps, char *report,
                             size_t report_bytes);
 
-/* Name of the interior kernel the context runs (for reports). */
+/* Name of the interior kernel lwacm_step runs (for reports). It begins with the class of
+ * LWACM_OPT_KERNEL, as bound: "generic_..." (1), "half_..." (5), "tiles2d_..." (6), "batch_..." for
+ * an ensemble. What follows says which kernel of the class:
+ *   half_d3q19_tma       the half-row TMA kernel; +nu_p_sum: after the pass that sums omega_p's
+ *                        density term; +scalar_rows / +scalar_rows_march: the passive scalar
+ *                        on its row-tiled kernel / on marching warps after it
+ *   half_d3q19_march     warps that march along z (nothing of the half-row kernel runs)
+ *   generic_d3q19_march  the same under kernel 1; +scalar_march: the scalar likewise after it
+ *   generic_d3q19, generic_d2q9  one node a thread, gathering; the scalar in the same kernel
+ *   tiles2d_d2q9_rows    warps that march along y; +cluster: calls of four steps and more in
+ *                        one launch of a thread-block cluster
+ *   tiles2d_d2q9_WxH     2D tiles
+ *   batch_rows_step, batch_rows_persistent  the D2Q9 march over an ensemble's strips
+ *   batch_step, batch_persistent, batch_tilesWxH_...  runs of nodes, 2D tiles
+ * Recorded runs (lwacm_forward_record) run the half-row kernel, the 30x14 (or chosen) tiles or
+ * the gather of the same class. */
 const char *lwacm_kernel_name(const lwacm_ctx *ctx);
 
 /* Release the context (host memory and CUDA graphs). Does not touch the bound

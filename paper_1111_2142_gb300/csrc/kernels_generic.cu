@@ -788,16 +788,9 @@ cudaError_t launch_step_generic_t(int Q, const void *in, void *out, const StepPa
     return cudaGetLastError();
 }
 
-cudaError_t launch_step_generic(int Q, int storage, const void *in, void *out,
-                                const StepParams &p, cudaStream_t st) {
-    // one node a thread gathering from global memory: 201 x 131 x 150 127 us a step, 60^3
-    // 10.6, marching warps 36 and 4.6; kept for what those do not do (omega_p, the scalar,
-    // D2Q9 with it, fewer than four rows) and for recorded runs
-    if (Q == 19 && rows3d_supported(p)) return launch_step_rows3d(storage, in, out, p, st);
-    return launch_step_gather(Q, storage, in, out, p, st);
-}
-
-cudaError_t launch_step_gather(int Q, int storage, const void *in, void *out, const StepParams &p, cudaStream_t st) {
+// 201 x 131 x 150 127 us a step, 60^3 10.6, marching warps 36 and 4.6; kept for what those do not
+// do (omega_p, the scalar, D2Q9 with it, fewer than four rows) and for recorded runs
+cudaError_t launch_step_generic(int Q, int storage, const void *in, void *out, const StepParams &p, cudaStream_t st) {
     switch (storage) {
         case STORE_F32: return launch_step_generic_t<float>(Q, in, out, p, st);
         case STORE_BF16: return launch_step_generic_t<__nv_bfloat16>(Q, in, out, p, st);

@@ -16,10 +16,8 @@ enum { XFER_F32 = 0, XFER_F64 = 3 };
 constexpr int kDiagBlocks = 152 * 2;  // fixed grid -> deterministic reduction order
 constexpr int kDiagValues = 9;
 
-cudaError_t launch_step_generic(int Q, int storage, const void *in, void *out,
-                                const StepParams &p, cudaStream_t st);
 // one node a thread gathering from global memory, whatever the scheme and shape
-cudaError_t launch_step_gather(int Q, int storage, const void *in, void *out, const StepParams &p, cudaStream_t st);
+cudaError_t launch_step_generic(int Q, int storage, const void *in, void *out, const StepParams &p, cudaStream_t st);
 cudaError_t launch_wall_pass(int Q, int storage, const void *in, void *out, const StepParams &p,
                              cudaStream_t st);
 // semi-implicit density pass (Eq. FDcompact_si) after the explicit step in -> out

@@ -42,7 +42,7 @@ struct lwacm_ctx {
     bool semi = false;        // semi-implicit pressure update (Eq. FDcompact_si)
     bool sr = false;          // BF16 / FP16 stores rounded stochastically (half-row kernel)
     bool no_cluster = false;  // the device does not take the cluster kernel
-    bool march = false;       // kernel 5, automatic choice: by warps that march along z (kernels_rows3.cu)
+    bool march = false;       // D3Q19, kernels 1 and 5: by warps that march along z (kernels_rows3.cu)
     bool recording = false;   // the steps of a recorded run (step_between)
     bool scalar_rows = false; // the passive scalar on its own kernel after the half-row flow kernel
     bool scalar_march = false;  // on its own marching kernel after the general flow kernel
@@ -195,21 +195,28 @@ void drop_graphs(lwacm_ctx *c) {
     }
 }
 
-// Interior kernel: the explicit choice if it supports the shape, else (automatic)
-// the half-row TMA kernel (D3Q19), then the 2D-tile kernel (D2Q9), then the
-// generic gather kernel, which supports everything. Returns false when an
-// explicit choice is not supported. Kernels that need the device are only
-// considered once a workspace is bound.
+// whether runs of steps go to one cluster (kernels_cluster2.cu): a small D2Q9 domain on the
+// marching kernel
+bool cluster_ok(const lwacm_ctx *c) {
+    return c->kernel == 6 && c->batch_shape == 0 && !c->semi && !c->no_cluster && cluster2d_supported(params(c));
+}
+
+// Interior kernel: the explicit choice if it supports the shape, else (automatic) kernel 5 (D3Q19:
+// the half-row TMA kernel or, where faster, warps that march along z), then kernel 6 (D2Q9: warps
+// that march along y, many steps in one cluster for a small domain, or the 2D tiles of
+// LWACM_OPT_BATCH_TILE), then kernel 1, which supports everything (the D3Q19 march where it applies,
+// else the gather). Returns false when an explicit choice is not supported. Kernels that need the
+// device are only considered once a workspace is bound.
 bool choose_kernel(lwacm_ctx *c) {
     if (c->nbatch) {
         c->kernel = 4;
         static const char *names[2][8] = {
             {"batch_step", "batch_tiles30x6_step", "batch_tiles30x14_step", "batch_tiles62x6_step",
-             "batch_tiles30x30_step", "batch_tiles62x14_step", "batch_tiles126x6_step", "batch_step"},
+             "batch_tiles30x30_step", "batch_tiles62x14_step", "batch_tiles126x6_step", "batch_rows_step"},
             {"batch_persistent", "batch_tiles30x6_persistent", "batch_tiles30x14_persistent",
              "batch_tiles62x6_persistent", "batch_tiles30x30_persistent", "batch_tiles62x14_persistent",
-             "batch_tiles126x6_persistent", "batch_persistent"}};
-        c->kname = names[c->batch_mode ? 1 : 0][c->batch_shape & 7];
+             "batch_tiles126x6_persistent", "batch_rows_persistent"}};
+        c->kname = names[c->batch_mode ? 1 : 0][c->batch_shape == 0 && c->Q == 9 ? 7 : c->batch_shape];
         return c->kernel_opt == 0 || c->kernel_opt == 1;
     }
     const StepParams p = params(c);
@@ -237,19 +244,29 @@ bool choose_kernel(lwacm_ctx *c) {
     if (c->kernel != 5) c->scalar_rows = false;
     StepParams flow = p;
     flow.scalar = 0;
-    c->scalar_march = p.scalar && c->Q == 19 && c->kernel == 1 && rows3d_supported(flow);
+    c->scalar_march = p.scalar && c->Q == 19 && c->kernel == 1 && dev && rows3d_supported(flow);
     // rows the half-row kernel takes, plain scheme: marching warps, which need no halves or
     // segments (us a step, half-row / march: 256^3 137 / 129, 256 x 128 x 128 39 / 35, 384 x 256 x
     // 256 278 / 178, 200 x 256 x 256 190 / 100), but for whole rows of one warp (128 x 256 x 256 65 /
     // 77) and for a cavity whose x walls the half-row kernel applies
-    c->march = c->kernel == 5 && c->kernel_opt == 0 && !c->sr && !c->scalar_rows && rows3d_supported(p) && c->nx != 128 &&
-               (c->bc == LWACM_BC_PERIODIC || !half_xwalls(p));
-    static const char *hname[2][2] = {{"half_d3q19_tma", "half_d3q19_tma+scalar_rows"},
-                                      {"half_d3q19_tma+nu_p_sum", "half_d3q19_tma+nu_p_sum+scalar_rows"}};
-    c->kname = c->march         ? "half_d3q19_march"
-               : c->kernel == 5 ? hname[p.sdelta != 0.f ? 1 : 0][c->scalar_rows ? 1 : 0]
-               : c->kernel == 6 ? (dev && c->batch_shape == 0 ? "tiles2d_d2q9_rows" : sname[c->batch_shape < 7 ? c->batch_shape : 0])
-                                : gname[c->Q == 19 ? 1 : 0];
+    if (c->kernel == 5)
+        c->march = c->kernel_opt == 0 && !c->sr && !c->scalar_rows && rows3d_supported(p) && c->nx != 128 &&
+                   (c->bc == LWACM_BC_PERIODIC || !half_xwalls(p));
+    else
+        c->march = c->kernel == 1 && c->Q == 19 && dev && rows3d_supported(flow);
+    // the first part names the class of LWACM_OPT_KERNEL, the rest what runs
+    if (c->kernel == 5) {
+        c->kname = c->march ? "half_d3q19_march" : "half_d3q19_tma";
+        if (p.sdelta != 0.f) c->kname += "+nu_p_sum";
+        if (c->scalar_rows) c->kname += c->nx == 128 ? "+scalar_rows" : "+scalar_rows_march";
+    } else if (c->kernel == 6) {
+        c->kname = !dev || c->batch_shape > 0 ? sname[c->batch_shape] : "tiles2d_d2q9_rows";
+        if (dev && cluster_ok(c)) c->kname += "+cluster";
+    } else {
+        c->kname = gname[c->Q == 19 ? 1 : 0];
+        if (c->march) c->kname += "_march";
+        if (c->scalar_march) c->kname += "+scalar_march";
+    }
     return ok;
 }
 
@@ -339,22 +356,19 @@ cudaError_t step_between(lwacm_ctx *c, const void *in, void *out, cudaStream_t s
     // is a sum that may cancel, and the marching kernels' other order of additions moved it by more
     // than 2e-5 in one of five random runs
     const bool rec = c->recording;
-    e = rec && c->kernel == 6        ? launch_step_tiles2d(c->Q, c->storage, c->batch_shape > 0 ? c->batch_shape : 2, in,
-                                                           out, p, st)
-                    : rec && c->kernel == 1 ? launch_step_gather(c->Q, c->storage, in, out, p, st)
-                    : c->march && !rec ? launch_step_rows3d(c->storage, in, out, p, st)
-                    : c->kernel == 5 ? launch_step_half(c->Q, c->storage, in, out, pf, st)
-                    : c->kernel == 6 && c->batch_shape == 0 ? launch_step_rows2d(c->storage, in, out, p, st)
-                    : c->kernel == 6 ? launch_step_tiles2d(c->Q, c->storage, c->batch_shape, in, out, p, st)
-                                     : launch_step_generic(c->Q, c->storage, in, out, pf, st);
+    const bool march = c->march && !rec;
+    e = march            ? launch_step_rows3d(c->storage, in, out, pf, st)
+        : c->kernel == 5 ? launch_step_half(c->Q, c->storage, in, out, pf, st)
+        : c->kernel == 6 && c->batch_shape == 0 && !rec ? launch_step_rows2d(c->storage, in, out, p, st)
+        : c->kernel == 6 ? launch_step_tiles2d(c->Q, c->storage, c->batch_shape > 0 ? c->batch_shape : 2, in, out, p, st)
+                         : launch_step_generic(c->Q, c->storage, in, out, pf, st);
     if (e != cudaSuccess) return e;
     // the D2Q9 and the marching D3Q19 kernels apply the wall rule themselves; the half-row
     // kernel the x-face walls of a cavity whose lid is not on an x face
-    const bool walls_done =
-        c->kernel == 6 || (!rec && (c->march || c->kernel == 1) && c->Q == 19 && rows3d_walls(p));
+    const bool walls_done = c->kernel == 6 || (march && rows3d_walls(p));
     if (c->bc != LWACM_BC_PERIODIC && !walls_done) {
         StepParams pw = p;
-        pw.xfaces_done = c->kernel == 5 && (rec || !c->march) && half_xwalls(p) ? 1 : 0;
+        pw.xfaces_done = c->kernel == 5 && !march && half_xwalls(p) ? 1 : 0;
         e = launch_wall_pass(c->Q, c->storage, in, out, pw, st);
     }
     if (e == cudaSuccess && p.sr_ctr && c->kernel == 5) e = launch_sr_tick(p.sr_ctr, st);
@@ -371,12 +385,9 @@ cudaError_t enqueue_step(lwacm_ctx *c, int cur, cudaStream_t st) {
     return step_between(c, bufp(c, cur), bufp(c, 1 - cur), st);
 }
 
-// whether n steps run on one cluster (kernels_cluster2.cu): a small D2Q9 domain on the marching
-// kernel. A launch costs 8 us, single steps 2.1 to 2.5 each where no graph is replayed (64^2: 4
-// steps 10.9 us against 15.7, 2 steps 12.0 against 13.7).
-bool on_cluster(const lwacm_ctx *c, long long n) {
-    return n >= 4 && !c->recording && c->kernel == 6 && c->batch_shape == 0 && !c->semi && !c->no_cluster && cluster2d_supported(params(c));
-}
+// whether n steps run on one cluster. A launch costs 8 us, single steps 2.1 to 2.5 each where no
+// graph is replayed (64^2: 4 steps 10.9 us against 15.7, 2 steps 12.0 against 13.7).
+bool on_cluster(const lwacm_ctx *c, long long n) { return n >= 4 && !c->recording && cluster_ok(c); }
 
 // the steps of a recorded run, while it lives; graphs of other steps are not replayed in it nor its own
 // after it (runs whose segments are shorter than a graph capture none)
