@@ -32,6 +32,7 @@ using rows2::Walls2;
 
 constexpr int kCtas = 16;       // CTAs of the cluster
 constexpr int kThreads = 1024;  // threads of a CTA at most
+constexpr int kMaxSmem = 227 * 1024;
 constexpr int kNodes = 1664;    // nodes of a CTA at most, one or two a thread: the marching kernel in
                                 // graphs catches up there (us a step over 256 steps, cluster / march:
                                 // 64^2 0.62 / 1.26, 128^2 1.05 / 1.46, 160^2 1.43 / 1.89, its cavity
@@ -284,28 +285,35 @@ template <int PER, typename T, bool WALLS, bool BULK, bool NUP>
 cudaError_t launch_k(const void *in, void *out, const Small2 &q, const Shape &s, int steps, cudaStream_t st) {
     auto kern = k_d2q9_cluster<PER, T, WALLS, BULK, NUP>;
     const size_t bytes = link_bytes(q.nx, s.nrows, NUP);
-    // opt in once per device: clusters of 16, the largest shared memory this kernel asks for
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = kCtas;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    // once per device: opt in to clusters of 16 and to the largest shared memory this kernel asks for,
+    // and see whether the device has room for such a cluster
     static DevSlots set;
     const int ok = per_device(set, [&] {
-        return cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
-                       cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) ==
-                           cudaSuccess
-                   ? 1
-                   : -1;
+        cfg.gridDim = dim3(kCtas);
+        cfg.blockDim = dim3(kThreads);
+        cfg.dynamicSmemBytes = kMaxSmem;
+        int clusters = 0;
+        const bool fits =
+            cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem) == cudaSuccess &&
+            cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg) == cudaSuccess && clusters > 0;
+        if (!fits) cudaGetLastError();
+        return fits ? 1 : -1;
     });
     if (ok < 1) return cudaErrorNotSupported;
-    cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)s.ctas);
     cfg.blockDim = dim3((unsigned)s.threads);
     cfg.dynamicSmemBytes = bytes;
     cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = (unsigned)s.ctas;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kern, (const T *)in, (T *)out, q, steps);
 }
 template <int PER, typename T>
@@ -328,7 +336,7 @@ cudaError_t launch_t(const void *in, void *out, const Small2 &q, const Shape &s,
 
 bool cluster2d_supported(const StepParams &p) {
     const Shape s = shape_of(p.nx, p.ny);
-    return !p.gfield && s.per > 0 && link_bytes(p.nx, s.nrows, p.sdelta != 0.f) <= 227 * 1024;
+    return !p.gfield && s.per > 0 && link_bytes(p.nx, s.nrows, p.sdelta != 0.f) <= kMaxSmem;
 }
 
 cudaError_t launch_cluster2d(int storage, const void *in, void *out, const StepParams &p, int steps, cudaStream_t st) {

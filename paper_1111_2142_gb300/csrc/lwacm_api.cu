@@ -987,11 +987,12 @@ lwacm_status lwacm_step(lwacm_ctx *c, long long n) {
         // caller that captures an even number into a graph of its own replays it on and on)
         const int to = c->cur ^ (m & 1);
         const cudaError_t e = launch_cluster2d(c->storage, bufp(c, c->cur), bufp(c, to), params(c), m, c->stream);
-        if (e != cudaSuccess) {  // refused before it ran (a device without clusters of this size)
-            cudaGetLastError();
+        if (e == cudaErrorNotSupported) {  // no room for a cluster of this size on this device
             c->no_cluster = true;
+            choose_kernel(c);
             break;
         }
+        CK(c, e, "cluster launch");
         c->cur = to;
         c->steps += m;
         left -= m;

@@ -100,3 +100,40 @@ def test_cluster_leaves_the_state_in_the_buffer_of_single_steps(lw, n):
             assert np.array_equal(a, b)
         ref.close()
     sim.close()
+
+
+def takes_cluster(shape, nu_p):
+    """The bounds of the cluster kernel: at most 1664 nodes and 227 KB of link arrays a CTA."""
+    ny, nx = shape
+    rows = -(-ny // min(ny, 16))
+    return rows * nx <= 1664 and 2 * (12 if nu_p else 8) * (rows + 2) * nx * 4 <= 227 * 1024
+
+
+# two nodes a thread: square, uneven rows, tall, two rows and one row a CTA up to the largest
+@pytest.mark.parametrize("storage", [0, 1, 2])
+@pytest.mark.parametrize("shape", [(160, 160), (165, 130), (255, 97), (175, 150), (17, 800), (16, 1100), (16, 1210)])
+def test_two_nodes_a_thread(lw, shape, storage):
+    assert takes_cluster(shape, False) and -(-shape[0] // 16) * shape[1] > 1024
+    both(lw, shape, 5, storage=storage)
+    both(lw, shape, 6, storage=storage, force=(1e-4, 2e-5))
+    both(lw, shape, 5, storage=storage, nu_p=0.1)
+    both(lw, shape, 5, storage=storage, bulk_gamma=0.4)
+    both(lw, shape, 6, storage=storage, bulk_gamma=0.3, nu_p=0.08)
+    both(lw, shape, 5, bc=1, storage=storage)
+    both(lw, shape, 5, bc=2, storage=storage, force=(1e-4, 0.0))
+
+
+@pytest.mark.parametrize("nu_p", [None, 0.1])
+@pytest.mark.parametrize("shape", SHAPES + [(160, 160), (17, 800), (16, 1210), (16, 1211), (176, 152)])
+def test_the_cluster_ran(lw, shape, nu_p):
+    """Where the domain is within its bounds the cluster takes the steps: the name keeps saying so
+    after them (a device that refused it would have fallen back to single steps)."""
+    ny, nx = shape
+    sim = lw.Lwacm(9, nx, ny, 1, 0.02)
+    if nu_p:
+        sim.set_option(lw.OPT_NU_P, nu_p)
+    sim.set_fields(*inputs.smooth_random(shape, seed=74, u_amp=0.05, d_amp=0.01))
+    sim.step(8)
+    sim.sync()
+    assert sim.kernel_name == "tiles2d_d2q9_rows" + ("+cluster" if takes_cluster(shape, nu_p) else "")
+    sim.close()
