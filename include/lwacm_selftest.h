@@ -53,6 +53,12 @@ int lwacm_selftest_round(const float *x_dev, float *out_dev, long long n, int st
 int lwacm_selftest_schedule(int cols, int nz, int ctas, int *grid, int *zc, int *kcls, int *items, long long cap,
                             long long *count);
 
+/* *count = how many CUDA graphs of steps a context (lwacm_ctx, lwacm.h) has captured since it was
+ * created, by lwacm_prepare, lwacm_step and lwacm_forward_record: a step graph is captured once and
+ * replayed until an option changes. Host only. Errors: LWACM_E_ARG (null pointer). */
+struct lwacm_ctx;
+int lwacm_selftest_graph_builds(const struct lwacm_ctx *ctx, long long *count);
+
 #ifdef __cplusplus
 }
 #endif

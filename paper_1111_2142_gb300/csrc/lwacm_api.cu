@@ -14,6 +14,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include "../../include/lwacm.h"
+#include "../../include/lwacm_selftest.h"
 #include "launch.h"
 #include "lwacm_core.cuh"
 
@@ -66,10 +67,11 @@ struct lwacm_ctx {
     // status
     lwacm_status sticky = LWACM_OK;
     std::string err;
-    // graphs: one per starting buffer parity
+    // graphs: one per starting buffer parity, those of recorded runs after those of other steps
     cudaStream_t cap_stream = nullptr;
-    cudaGraphExec_t gexec[2] = {nullptr, nullptr};
-    int gchunk[2] = {0, 0};
+    cudaGraphExec_t gexec[4] = {nullptr, nullptr, nullptr, nullptr};
+    int gchunk[4] = {0, 0, 0, 0};
+    long long builds = 0;  // graphs captured so far
     int kernel = 1;  // 1 generic, 4 batch, 5 half-row TMA, 6 D2Q9 2D tiles (2 and 3: retired
                      // row-tiled kernels, superseded by 5)
     std::string kname = "none";
@@ -188,7 +190,7 @@ StepParams params(const lwacm_ctx *c) {
 }
 
 void drop_graphs(lwacm_ctx *c) {
-    for (int k = 0; k < 2; ++k) {
+    for (int k = 0; k < 4; ++k) {
         if (c->gexec[k]) cudaGraphExecDestroy(c->gexec[k]);
         c->gexec[k] = nullptr;
         c->gchunk[k] = 0;
@@ -389,20 +391,14 @@ cudaError_t enqueue_step(lwacm_ctx *c, int cur, cudaStream_t st) {
 // graph is replayed (64^2: 4 steps 10.9 us against 15.7, 2 steps 12.0 against 13.7).
 bool on_cluster(const lwacm_ctx *c, long long n) { return n >= 4 && !c->recording && cluster_ok(c); }
 
-// the steps of a recorded run, while it lives; graphs of other steps are not replayed in it nor its own
-// after it (runs whose segments are shorter than a graph capture none)
+// the steps of a recorded run, while it lives: other kernels (step_between) and graphs of its own
 struct Recording {
     lwacm_ctx *c;
-    bool graphs;
-    Recording(lwacm_ctx *c_, long long seg) : c(c_), graphs(c_->graph_chunk > 0 && seg >= c_->graph_chunk) {
-        c->recording = true;
-        if (graphs) drop_graphs(c);
-    }
-    ~Recording() {
-        c->recording = false;
-        if (graphs) drop_graphs(c);
-    }
+    explicit Recording(lwacm_ctx *c_) : c(c_) { c->recording = true; }
+    ~Recording() { c->recording = false; }
 };
+// the graph slot of steps that start in the current buffer
+int graph_slot(const lwacm_ctx *c) { return c->cur + (c->recording ? 2 : 0); }
 
 // whether n arrays lie in the current GPU's own memory
 bool all_local(const void *const *p, int n) {
@@ -453,7 +449,12 @@ lwacm_status ready(lwacm_ctx *c, bool need_fields) {
     return LWACM_OK;
 }
 
-lwacm_status build_graph(lwacm_ctx *c, int parity, int chunk) {
+lwacm_status build_graph(lwacm_ctx *c, int chunk) {
+    const int parity = c->cur, slot = graph_slot(c);
+    if (c->gexec[slot]) {
+        cudaGraphExecDestroy(c->gexec[slot]);
+        c->gexec[slot] = nullptr;
+    }
     if (!c->cap_stream) CK(c, cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking), "stream create");
     CK(c, cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal), "begin capture");
     int cur = parity;
@@ -473,8 +474,9 @@ lwacm_status build_graph(lwacm_ctx *c, int parity, int chunk) {
     cudaError_t ie = cudaGraphInstantiate(&ex, g, 0);
     cudaGraphDestroy(g);
     if (ie != cudaSuccess) return cuda_fail(c, ie, "graph instantiate");
-    c->gexec[parity] = ex;
-    c->gchunk[parity] = chunk;
+    ++c->builds;
+    c->gexec[slot] = ex;
+    c->gchunk[slot] = chunk;
     return LWACM_OK;
 }
 
@@ -955,13 +957,9 @@ lwacm_status lwacm_prepare(lwacm_ctx *c, long long n) {
     if (c->nbatch && c->batch_mode == 1) return LWACM_OK;  // one persistent launch, no graph
     if (on_cluster(c, n)) return LWACM_OK;
     if (chunk <= 0 || n < chunk) return LWACM_OK;
-    const int par = c->cur;
-    if (c->gexec[par] && c->gchunk[par] == chunk) return LWACM_OK;
-    if (c->gexec[par]) {
-        cudaGraphExecDestroy(c->gexec[par]);
-        c->gexec[par] = nullptr;
-    }
-    return build_graph(c, par, chunk);
+    const int slot = graph_slot(c);
+    if (c->gexec[slot] && c->gchunk[slot] == chunk) return LWACM_OK;
+    return build_graph(c, chunk);
 }
 
 lwacm_status lwacm_step(lwacm_ctx *c, long long n) {
@@ -1000,17 +998,13 @@ lwacm_status lwacm_step(lwacm_ctx *c, long long n) {
     const int chunk = c->graph_chunk;
     if (chunk > 0 && left >= chunk) {
         // graphs are replayed on the bound stream; capture needs a private stream
-        const int par = c->cur;
-        if (!c->gexec[par] || c->gchunk[par] != chunk) {
-            if (c->gexec[par]) {
-                cudaGraphExecDestroy(c->gexec[par]);
-                c->gexec[par] = nullptr;
-            }
-            s = build_graph(c, par, chunk);
+        const int slot = graph_slot(c);
+        if (!c->gexec[slot] || c->gchunk[slot] != chunk) {
+            s = build_graph(c, chunk);
             if (s != LWACM_OK) return s;
         }
         while (left >= chunk) {
-            CK(c, cudaGraphLaunch(c->gexec[par], c->stream), "graph launch");
+            CK(c, cudaGraphLaunch(c->gexec[slot], c->stream), "graph launch");
             left -= chunk;
             c->steps += chunk;  // chunk is even: parity unchanged
         }
@@ -1174,7 +1168,7 @@ lwacm_status lwacm_forward_record(lwacm_ctx *c, long long T, int stride, void *w
     c->adj_bytes = bytes;
     const size_t sb = (size_t)c->Nal * 4 * c->nf;
     c->rec_last_kept = false;
-    const Recording rec(c, L.S);
+    const Recording rec(c);
     for (long long k = 0; k < L.K; ++k) {
         char *ck = c->adj + L.ckpt + k * L.state;
         CK(c, cudaMemcpyAsync(ck, bufp(c, c->cur), sb, cudaMemcpyDeviceToDevice, c->stream), "checkpoint copy");
@@ -1224,7 +1218,7 @@ lwacm_status lwacm_backward(lwacm_ctx *c, const void *ld, const void *lux, const
     CK(c, launch_convert_in_fields(STORE_F32, dtype, lin, c->nf, lam0, c->Nal, c->N, c->stream), "lambda in");
     CK(c, cudaMemsetAsync(total, 0, 16, c->stream), "clear dnu");
     const StepParams p = params(c);
-    const Recording rec(c, 0);  // recomputed segments; no graph
+    const Recording rec(c);  // recomputed segments
     int cur = 0;
     for (long long k = L.K - 1; k >= 0; --k) {
         const long long t0 = k * L.S;
@@ -1375,6 +1369,12 @@ lwacm_status lwacm_autotune(lwacm_ctx *c, const char *cache_path, int trial_step
         r += "]}";
         std::snprintf(report, report_bytes, "%s", r.c_str());
     }
+    return LWACM_OK;
+}
+
+int lwacm_selftest_graph_builds(const lwacm_ctx *c, long long *count) {
+    if (!c || !count) return LWACM_E_ARG;
+    *count = c->builds;
     return LWACM_OK;
 }
 
