@@ -372,8 +372,9 @@ const char *lwacm_last_error(const lwacm_ctx *ctx);
  * stream; the call synchronises.
  *
  * cache_path (or NULL): a JSON file mapping a problem key (lattice, storage, boundary,
- * shape or the ensemble's sizes and viscosities, forcing, SM count and compute
- * capability) to the chosen configuration. On a hit nothing is timed and the
+ * shape or the ensemble's sizes and viscosities, forcing, SM count, compute
+ * capability and the generation of the kernels, so that an entry measured with other
+ * kernels is not taken) to the chosen configuration. On a hit nothing is timed and the
  * recorded choice is applied; on a miss the measured choice is added (written to a
  * temporary file renamed over the cache). report (or NULL): receives a one-line JSON
  * record (key, "cache" or "measured", the choice, every candidate's time), cut to

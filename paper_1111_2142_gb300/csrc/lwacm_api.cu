@@ -494,8 +494,13 @@ void fnv(uint64_t &h, const void *v, size_t n) {
     }
 }
 
+// Generation of the kernels the candidates stand for. An entry measured with other kernels would pin
+// a choice that was the fastest then (a 2D tile, where the marching kernel now is), so the
+// generation is part of the key: to be raised with each change that can move the choice.
+constexpr int kKernels = 2;
+
 // problem key: lattice, storage, boundary, shape (or the ensemble's sizes and
-// viscosities, hashed), forcing, and the device (SM count, compute capability)
+// viscosities, hashed), forcing, the device (SM count, compute capability) and the kernels
 std::string tune_key(const lwacm_ctx *c) {
     int dev = 0, sms = 0, mj = 0, mn = 0;
     cudaGetDevice(&dev);
@@ -511,12 +516,12 @@ std::string tune_key(const lwacm_ctx *c) {
             fnv(h, &d.nz, sizeof d.nz);
             fnv(h, &d.s, sizeof d.s);
         }
-        std::snprintf(buf, sizeof buf, "lattice=%d;storage=%d;batch=%d;nodes=%lld;domains=%016llx;sm=%d;cc=%d.%d",
-                      c->Q, c->storage, c->nbatch, c->N, (unsigned long long)h, sms, mj, mn);
+        std::snprintf(buf, sizeof buf, "lattice=%d;storage=%d;batch=%d;nodes=%lld;domains=%016llx;sm=%d;cc=%d.%d;kernels=%d",
+                      c->Q, c->storage, c->nbatch, c->N, (unsigned long long)h, sms, mj, mn, kKernels);
     } else {
         const bool forced = c->force[0] != 0 || c->force[1] != 0 || c->force[2] != 0 || c->ff_active;
-        std::snprintf(buf, sizeof buf, "lattice=%d;storage=%d;bc=%d;nx=%d;ny=%d;nz=%d;force=%d;sm=%d;cc=%d.%d", c->Q,
-                      c->storage, c->bc, c->nx, c->ny, c->nz, forced ? 1 : 0, sms, mj, mn);
+        std::snprintf(buf, sizeof buf, "lattice=%d;storage=%d;bc=%d;nx=%d;ny=%d;nz=%d;force=%d;sm=%d;cc=%d.%d;kernels=%d",
+                      c->Q, c->storage, c->bc, c->nx, c->ny, c->nz, forced ? 1 : 0, sms, mj, mn, kKernels);
     }
     return buf;
 }

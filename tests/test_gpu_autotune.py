@@ -87,3 +87,27 @@ def test_single_domain_autotune_and_unreadable_cache(lw, tmp_path):
     assert eu < 1e-5
     assert rep["key"] in json.loads(cache.read_text())
     sim.close()
+
+
+@pytest.mark.parametrize("kind", ["single", "batch"])
+def test_entries_of_other_kernels_are_not_taken(lw, tmp_path, kind):
+    """A cache written before the kernels changed names none of their generation: its entry is
+    left alone and the candidates are timed."""
+    cache = tmp_path / "tune.json"
+
+    def new():
+        return lw.Lwacm(lw.D2Q9, 300, 200, 1, 0.01) if kind == "single" else \
+            lw.LwacmBatch(lw.D2Q9, [(40, 30), (33, 61)], [0.01, 0.02])
+
+    sim = new()
+    key = sim.autotune(steps=8)["key"]
+    sim.close()
+    old = key[:key.rindex(";kernels=")]
+    cache.write_text('{\n"%s": {"kernel": %d, "tile": 4, "mode": 0, "us_per_step": 0.001}\n}\n'
+                     % (old, 6 if kind == "single" else 0))
+    sim = new()
+    rep = sim.autotune(cache=cache, steps=8)
+    assert rep["source"] == "measured" and rep["key"] == key
+    entries = json.loads(cache.read_text())
+    assert old in entries and key in entries
+    sim.close()
