@@ -89,7 +89,8 @@ enum {
                                   0 disables graphs; default 64) */
     LWACM_OPT_KERNEL = 9,  /* interior kernel: 0 = automatic choice (default),
                               1 = general kernel (any size and option; the plain
-                              D3Q19 scheme by warps that march along z, else a gather),
+                              D3Q19 scheme by warps that march along z but for
+                              domains of a few columns or rows, else a gather),
                               5 = D3Q19 half-row TMA kernel
                               (needs the plain scheme, with or without a constant
                               acceleration but not a force field, nx = 128, 256 or

@@ -789,7 +789,8 @@ cudaError_t launch_step_generic_t(int Q, const void *in, void *out, const StepPa
 }
 
 // 201 x 131 x 150 127 us a step, 60^3 10.6, marching warps 36 and 4.6; kept for what those do not
-// do (omega_p, the scalar, D2Q9 with it, fewer than four rows) and for recorded runs
+// do (omega_p, the scalar with it, D2Q9, fewer than four rows), for narrow domains
+// (rows3d_pays) and for recorded runs
 cudaError_t launch_step_generic(int Q, int storage, const void *in, void *out, const StepParams &p, cudaStream_t st) {
     switch (storage) {
         case STORE_F32: return launch_step_generic_t<float>(Q, in, out, p, st);

@@ -554,6 +554,25 @@ bool rows3d_supported(const StepParams &p) {
     return p.ny >= kTile && (long long)p.nx * p.ny < (1LL << 30) && p.sdelta == 0.f && !p.scalar && !p.bulk;
 }
 
+// Whether the march takes less than the gather (with the scalar: its two kernels less than the
+// gather's one). A warp works on 30 columns and a CTA on 16 rows whatever the domain has, so a
+// narrow one pays for `slots` nodes and a gather only for its own: picoseconds a step, fitted to 200
+// shapes of 1 to 95 columns and 5 to 1000 rows (us a step, gather / march: 2 x 256 x 256 8.4 /
+// 15.5, 4 x 256 x 256 13.7 / 15.5, 5 x 256 x 256 16.3 / 15.5, 6 x 6 x 10000 18.1 / 33.8, 14 x 6 x
+// 10000 36.4 / 33.8, 1 x 64 x 64 4.7 / 3.6; with the scalar 4 x 256 x 256 15.3 / 28.0, 8 x 256 x 256
+// 27.6 / 28.1, 2 x 24 x 24 5.4 / 5.1). The gather of a walled domain has the wall pass after it, the
+// march not (a channel of 2 x 256 x 256 15.4 / 19.8, of 4 x 256 x 256 19.8 / 20.0, of 8 x 6 x 10000
+// 34.7 / 41.9; a cavity of 3 x 256 x 256 20.1 / 23.1, of 6 x 6 x 10000 76.7 / 50.1).
+bool rows3d_pays(const StepParams &p) {
+    const double n = (double)p.N, cols = (double)((p.nx - 1) / kStrip + 1) * kStrip;
+    const double slots = cols * ((p.ny - 1) / (kTile * kWarps) + 1) * (kTile * kWarps) * p.nz;
+    if (p.scalar) return 13.0 * cols * ((p.ny - 1) / kTile + 1) * kTile * p.nz < 45.0 * n + 0.4e6;
+    if (rows3d_walls(p))
+        return (p.bc == BC_CAVITY ? 11.0 * slots - 2000.0 * n / p.ny : 9.0 * slots - 140.0 * n / p.ny) <
+               38.0 * n + 9.5e6;
+    return (p.gfield ? 8.0 : 7.0) * slots < 38.0 * n + 2.8e6;
+}
+
 // Walls applied in the kernel (no wall pass after it), without a force field, up to 2^20 nodes:
 // the bounces take registers (232: two CTAs a SM instead of four) and instructions in every
 // boundary warp, a wall pass 5 to 8 us a step (kernel and pass / walls in the kernel: the 60^3

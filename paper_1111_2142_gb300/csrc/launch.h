@@ -105,6 +105,8 @@ bool cluster2d_supported(const StepParams &p);
 cudaError_t launch_cluster2d(int storage, const void *in, void *out, const StepParams &p, int steps, cudaStream_t st);
 // the plain D3Q19 scheme by warps that march along z (kernels_rows3.cu), any size
 bool rows3d_supported(const StepParams &p);
+// whether it (with the scalar: with launch_scalar_march after it) is the faster one, not the gather
+bool rows3d_pays(const StepParams &p);
 // runs of planes a column of strips and tiles is cut into, for a GPU that holds `room` CTAs
 int rows3d_runs(long long cols, int nz, int room);
 // the passive scalar (Eq. ACM2.0t) the same way (kernels_scalar3.cu), after the flow kernel on the

@@ -246,7 +246,7 @@ bool choose_kernel(lwacm_ctx *c) {
     if (c->kernel != 5) c->scalar_rows = false;
     StepParams flow = p;
     flow.scalar = 0;
-    c->scalar_march = p.scalar && c->Q == 19 && c->kernel == 1 && dev && rows3d_supported(flow);
+    c->scalar_march = p.scalar && c->Q == 19 && c->kernel == 1 && dev && rows3d_supported(flow) && rows3d_pays(p);
     // rows the half-row kernel takes, plain scheme: marching warps, which need no halves or
     // segments (us a step, half-row / march: 256^3 137 / 129, 256 x 128 x 128 39 / 35, 384 x 256 x
     // 256 278 / 178, 200 x 256 x 256 190 / 100), but for whole rows of one warp (128 x 256 x 256 65 /
@@ -255,7 +255,7 @@ bool choose_kernel(lwacm_ctx *c) {
         c->march = c->kernel_opt == 0 && !c->sr && !c->scalar_rows && rows3d_supported(p) && c->nx != 128 &&
                    (c->bc == LWACM_BC_PERIODIC || !half_xwalls(p));
     else
-        c->march = c->kernel == 1 && c->Q == 19 && dev && rows3d_supported(flow);
+        c->march = c->kernel == 1 && c->Q == 19 && dev && rows3d_supported(flow) && rows3d_pays(p);
     // the first part names the class of LWACM_OPT_KERNEL, the rest what runs
     if (c->kernel == 5) {
         c->kname = c->march ? "half_d3q19_march" : "half_d3q19_tma";

@@ -88,3 +88,41 @@ def test_march_carries_extreme_values(lw, field, bad):
         assert np.array_equal(np.isfinite(x), np.isfinite(y))
         ok = np.isfinite(y) & (np.abs(y) < 1e3)
         assert np.allclose(x[ok], y[ok], rtol=0, atol=1e-3)
+
+
+# narrow domains of many nodes, each side of the line between the gather and the march (with the
+# scalar, in a channel, a force field): the kernel and its fields
+@pytest.mark.parametrize("shape,kw,name", [
+    ((256, 256, 2), {}, "generic_d3q19"), ((256, 256, 4), {}, "generic_d3q19"), ((256, 256, 6), {}, "generic_d3q19_march"),
+    ((10000, 6, 6), {}, "generic_d3q19"), ((10000, 6, 15), {}, "generic_d3q19_march"),
+    ((64, 64, 1), {}, "generic_d3q19_march"), ((256, 256, 3), dict(bc=2), "generic_d3q19"),
+    ((256, 256, 5), dict(bc=2), "generic_d3q19_march"), ((256, 256, 3), dict(bc=1), "generic_d3q19"),
+    ((1000, 6, 6), dict(bc=1), "generic_d3q19_march"),
+    ((256, 256, 4), dict(g=True), "generic_d3q19"), ((256, 256, 5), dict(scalar=True), "generic_d3q19"),
+    ((256, 256, 10), dict(scalar=True), "generic_d3q19_march+scalar_march"),
+    ((1000, 16, 4), dict(scalar=True), "generic_d3q19"), ((24, 24, 4), dict(scalar=True), "generic_d3q19_march+scalar_march")])
+def test_narrow_domains(lw, shape, kw, name):
+    nz, ny, nx = shape
+    f = inputs.smooth_random(shape, seed=57, u_amp=0.05, d_amp=0.01)
+    bc, lid = kw.get("bc", 0), (0.05, -0.03, 0.01) if kw.get("bc") else None
+    g = [1e-4 * c for c in inputs.smooth_random(shape, seed=58, u_amp=1.0, d_amp=1.0)[1:4]] if kw.get("g") else None
+    sim = lw.Lwacm(19, nx, ny, nz, 0.02, bc, lid=lid, force_field=g is not None, scalar_alpha=0.03 if kw.get("scalar") else None)
+    sim.set_fields(*f)
+    if g is not None:
+        sim.set_force_field(*g)
+    T0 = 1.0 + 0.2 * f[0] / float(np.max(np.abs(f[0])))
+    if kw.get("scalar"):
+        sim.set_scalar(T0)
+    assert sim.kernel_name == name
+    sim.step(3)
+    got = sim.get_fields()
+    if kw.get("scalar"):
+        ref = oracle.step_scalar(19, *f, T=T0, nu=0.02, alpha=0.03, nsteps=3)
+        assert float(np.max(np.abs(sim.get_scalar() - ref[-1]))) < 2e-6
+        ref = ref[:-1]
+    elif g is not None:
+        ref = oracle.step_force_field(19, *f, nu=0.02, g=g, nsteps=3)
+    else:
+        ref = oracle.step(19, *f, nu=0.02, nsteps=3, bc=bc, lid=lid)
+    within(got, ref)
+    sim.close()
