@@ -42,9 +42,8 @@ namespace {
 constexpr int kTile = 256;
 constexpr int kBarrierPolls = 1 << 21;  // with 256 ns back-off: well under a second
 
-template <int Q, typename T>
-__device__ __forceinline__ void tile_update(const T *__restrict__ in, T *__restrict__ out,
-                                            const BatchParams &bp, long long t) {
+template <int Q, bool RO, typename T>
+__device__ __forceinline__ void tile_update(const T *in, T *out, const BatchParams &bp, long long t) {
     const BatchTile tile = bp.tiles[t];
     const BatchDomain dm = bp.doms[tile.dom];
     const long long k = tile.start + threadIdx.x;
@@ -87,7 +86,7 @@ __device__ __forceinline__ void tile_update(const T *__restrict__ in, T *__restr
         y = (int)(r % dm.ny);
         z = (int)(r / dm.ny);
     }
-    node_update<Q, false>(in + dm.off, out + dm.off, p, x, y, z);
+    node_update<Q, false, false, false, false, RO>(in + dm.off, out + dm.off, p, x, y, z);
 }
 
 // ---- 2D tiles (D2Q9) -------------------------------------------------------------
@@ -135,9 +134,10 @@ struct Force2 {
 // W_p becomes (w_p rho + kappa_p / 3) (c_p.u); the trace is normalised by the
 // zeroth moment of the distribution built with a (the density before the sdelta
 // terms).
-template <int TW, int TH, typename T, bool WALLS = false, bool BULK = false, bool NUP = false>
-__device__ __forceinline__ void tile2_core(const T *__restrict__ in, T *__restrict__ out, long long base, int nx,
-                                           int ny, long long fstride, float s, float a, int x0, int y0,
+// RO: `in` is not written while the kernel runs (ldx).
+template <int TW, int TH, typename T, bool WALLS = false, bool BULK = false, bool NUP = false, bool RO = true>
+__device__ __forceinline__ void tile2_core(const T *in, T *out, long long base, int nx, int ny, long long fstride,
+                                           float s, float a, int x0, int y0,
                                            float (*G)[(TW + 2) * (TH + 2)], const Walls2 &wl = Walls2{},
                                            const Force2 &fc = Force2{}, float gamma = 0.f,
                                            float (*O)[(TW + 2) * (TH + 2)] = nullptr, float sdelta = 0.f) {
@@ -159,7 +159,7 @@ __device__ __forceinline__ void tile2_core(const T *__restrict__ in, T *__restri
         if (y < 0) y += ny;
     }
     const long long k = base + (long long)y * nx + x;
-    const float d = ldf(in + k), u = ldf(in + fstride + k), v = ldf(in + 2 * fstride + k);
+    const float d = ldx<RO>(in + k), u = ldx<RO>(in + fstride + k), v = ldx<RO>(in + 2 * fstride + k);
     const float rho = 1.f + d;
     const float K = fmaf(-1.5f * rho, fmaf(u, u, v * v), d);  // d - 3/2 rho |u|^2
     const float nu = s * (1.f / 18.f);
@@ -177,7 +177,7 @@ __device__ __forceinline__ void tile2_core(const T *__restrict__ in, T *__restri
         // (they sum to 0 in mass and momentum and to 2 rho h in the trace)
         float cax = 0.f, cdg = 0.f, oax = 0.f, odg = 0.f, kax = 0.f, kdg = 0.f;
         if (BULK) {
-            const float h = 0.5f * gamma * ldf(in + 3 * fstride + k), rh = rho * h;
+            const float h = 0.5f * gamma * ldx<RO>(in + 3 * fstride + k), rh = rho * h;
             const float P = fmaf(u, u, fmaf(v, v, 2.f / 3.f));
             cax = 0.5f * rh * (1.f - P - h);
             cdg = 0.25f * rh * (h + P);
@@ -273,12 +273,13 @@ __device__ __forceinline__ void tile2_core(const T *__restrict__ in, T *__restri
     __syncthreads();  // G is rewritten by the next tile
 }
 
-template <int TW, int TH, typename T>
-__device__ __forceinline__ void tile2_update(const T *__restrict__ in, T *__restrict__ out, const BatchParams &bp,
-                                             long long t, float (*G)[(TW + 2) * (TH + 2)]) {
+template <int TW, int TH, bool RO, typename T>
+__device__ __forceinline__ void tile2_update(const T *in, T *out, const BatchParams &bp, long long t,
+                                             float (*G)[(TW + 2) * (TH + 2)]) {
     const BatchTile2 tile = bp.tiles2[t];
     const BatchDomain dm = bp.doms[tile.dom];
-    tile2_core<TW, TH, T>(in, out, dm.off, dm.nx, dm.ny, bp.fstride, dm.s, dm.a, tile.x0, tile.y0, G);
+    tile2_core<TW, TH, T, false, false, false, RO>(in, out, dm.off, dm.nx, dm.ny, bp.fstride, dm.s, dm.a, tile.x0,
+                                                   tile.y0, G);
 }
 
 // one D2Q9 domain, walls included (no separate wall pass); tiles numbered row-major
@@ -301,7 +302,7 @@ template <int TW, int TH, typename T>
 __global__ void __launch_bounds__((TW + 2) * (TH + 2)) k_batch_tiles(const T *__restrict__ in, T *__restrict__ out,
                                                                     BatchParams bp) {
     __shared__ float G[8][(TW + 2) * (TH + 2)];
-    for (long long t = blockIdx.x; t < bp.ntiles; t += gridDim.x) tile2_update<TW, TH, T>(in, out, bp, t, G);
+    for (long long t = blockIdx.x; t < bp.ntiles; t += gridDim.x) tile2_update<TW, TH, true>(in, out, bp, t, G);
 }
 
 // D2Q9, shape 0: one item of the table by one warp (rows2.cuh). In the persistent form
@@ -329,7 +330,7 @@ __global__ void __launch_bounds__(32 * rows_warps(NS)) k_batch_rows(const T *in,
 template <int Q, typename T>
 __global__ void __launch_bounds__(kTile) k_batch_step(const T *__restrict__ in, T *__restrict__ out,
                                                       BatchParams bp) {
-    for (long long t = blockIdx.x; t < bp.ntiles; t += gridDim.x) tile_update<Q, T>(in, out, bp, t);
+    for (long long t = blockIdx.x; t < bp.ntiles; t += gridDim.x) tile_update<Q, true>(in, out, bp, t);
 }
 
 // Grid-wide barrier number `gen` (1, 2, ...): arrive on a counter, the last CTA
@@ -363,6 +364,8 @@ __device__ bool grid_barrier(const BatchParams &bp, unsigned gen) {
     return ok_s != 0;
 }
 
+// The persistent forms read with ordinary loads what other CTAs wrote before the barrier: the
+// read-only path is for data that nobody writes during the kernel.
 template <int Q, typename T>
 __global__ void __launch_bounds__(kTile) k_batch_persistent(T *buf0, T *buf1, BatchParams bp,
                                                             long long nsteps, int parity) {
@@ -370,7 +373,7 @@ __global__ void __launch_bounds__(kTile) k_batch_persistent(T *buf0, T *buf1, Ba
         const int cur = (int)((parity + s) & 1);
         const T *in = cur ? buf1 : buf0;
         T *out = cur ? buf0 : buf1;
-        for (long long t = blockIdx.x; t < bp.ntiles; t += gridDim.x) tile_update<Q, T>(in, out, bp, t);
+        for (long long t = blockIdx.x; t < bp.ntiles; t += gridDim.x) tile_update<Q, false>(in, out, bp, t);
         if (s + 1 < nsteps) {
             // test hook: CTA 0 leaves without arriving, so the others' waits run out
             if (bp.withhold_step == s && blockIdx.x == 0) return;
@@ -403,7 +406,7 @@ __global__ void __launch_bounds__((TW + 2) * (TH + 2)) k_batch_tiles_persistent(
         const int cur = (int)((parity + s) & 1);
         const T *in = cur ? buf1 : buf0;
         T *out = cur ? buf0 : buf1;
-        for (long long t = blockIdx.x; t < bp.ntiles; t += gridDim.x) tile2_update<TW, TH, T>(in, out, bp, t, G);
+        for (long long t = blockIdx.x; t < bp.ntiles; t += gridDim.x) tile2_update<TW, TH, false>(in, out, bp, t, G);
         if (s + 1 < nsteps) {
             if (bp.withhold_step == s && blockIdx.x == 0) return;
             if (!grid_barrier(bp, (unsigned)(s + 1))) return;

@@ -70,6 +70,15 @@ __device__ __forceinline__ float ldf(const __nv_bfloat16 *p) { return __bfloat16
 __device__ __forceinline__ float ldf(const __half *p) { return __half2float(__ldg(p)); }
 __device__ __forceinline__ float ldf(const double *p) { return (float)__ldg(p); }
 
+// RO: through the read-only path, for data that nobody writes while the kernel runs; else an ordinary load
+__device__ __forceinline__ float to_f32(float v) { return v; }
+__device__ __forceinline__ float to_f32(__nv_bfloat16 v) { return __bfloat162float(v); }
+__device__ __forceinline__ float to_f32(__half v) { return __half2float(v); }
+template <bool RO, typename T>
+__device__ __forceinline__ float ldx(const T *p) {
+    return RO ? ldf(p) : to_f32(*p);
+}
+
 __device__ __forceinline__ void stf(float *p, float v) { *p = v; }
 __device__ __forceinline__ void stf(__nv_bfloat16 *p, float v) { *p = __float2bfloat16_rn(v); }
 __device__ __forceinline__ void stf(__half *p, float v) { *p = __float2half_rn(v); }

@@ -30,15 +30,16 @@ namespace lwacm {
 // moment of the updated distribution (the new density unless NUP). With NUP as
 // well the density pre-combines the increment with a_p: (a - a_p) sum_i Df^o_i =
 // (sdelta/3) sum_i Df^o_i more; the momentum and the trace keep a.
-template <int Q, bool WALLS, bool NUP = false, bool SC = false, bool BULK = false, typename T>
-__device__ __forceinline__ void node_update(const T *__restrict__ in, T *__restrict__ out,
-                                            const StepParams &p, int x, int y, int z) {
+//
+// RO: `in` is not written while the kernel runs (ldx).
+template <int Q, bool WALLS, bool NUP = false, bool SC = false, bool BULK = false, bool RO = true, typename T>
+__device__ __forceinline__ void node_update(const T *in, T *out, const StepParams &p, int x, int y, int z) {
     using L = Lat<Q>;
     const long long k = ((long long)z * p.ny + y) * p.nx + x;
     const T *Din = in, *Uin = in + p.fstride, *Vin = in + 2 * p.fstride,
             *Win = in + 3 * p.fstride;
-    const float dx = ldf(Din + k), ux = ldf(Uin + k), uy = ldf(Vin + k);
-    const float uz = (Q == 19) ? ldf(Win + k) : 0.f;
+    const float dx = ldx<RO>(Din + k), ux = ldx<RO>(Uin + k), uy = ldx<RO>(Vin + k);
+    const float uz = (Q == 19) ? ldx<RO>(Win + k) : 0.f;
     const float rx = 1.f + dx;
     const float qx = fmaf(ux, ux, fmaf(uy, uy, uz * uz));
     float dd = 0.f, jx = 0.f, jy = 0.f, jz = 0.f, dsp = 0.f, ts = 0.f, trs = 0.f, dfos = 0.f;
@@ -63,8 +64,8 @@ __device__ __forceinline__ void node_update(const T *__restrict__ in, T *__restr
         sy = sy < 0 ? sy + p.ny : (sy >= p.ny ? sy - p.ny : sy);
         sz = sz < 0 ? sz + p.nz : (sz >= p.nz ? sz - p.nz : sz);
         const long long s = outside ? k : ((long long)sz * p.ny + sy) * p.nx + sx;
-        const float ds = ldf(Din + s), us = ldf(Uin + s), vs = ldf(Vin + s);
-        const float ws = (Q == 19) ? ldf(Win + s) : 0.f;
+        const float ds = ldx<RO>(Din + s), us = ldx<RO>(Uin + s), vs = ldx<RO>(Vin + s);
+        const float ws = (Q == 19) ? ldx<RO>(Win + s) : 0.f;
         float g;
         if (!outside) {
             const float e = cx * us + cy * vs + cz * ws;
@@ -72,13 +73,13 @@ __device__ __forceinline__ void node_update(const T *__restrict__ in, T *__restr
             g = link_g(L::w(i), ds, 1.f + ds, e, q, p.s);
             if (NUP) dsp = fmaf(L::w(i) * (1.f + ds), e, dsp);  // sum of w rho e
             if (SC) {
-                const float tsrc = ldf(Tin + s);
+                const float tsrc = ldx<RO>(Tin + s);
                 const float even = tsrc + fmaf(4.5f * e, e, -1.5f * q);
                 ts = fmaf(L::w(i), fmaf(omt, even, 3.f * tsrc * e), ts);
             }
             if (BULK) {
                 const float pxx = fmaf(us, us, 1.f / 3.f), pyy = fmaf(vs, vs, 1.f / 3.f);
-                const float h = 0.5f * p.gamma * ldf(Tin + s);
+                const float h = 0.5f * p.gamma * ldx<RO>(Tin + s);
                 const float A = cx == 0 ? 1.f - pxx : 0.5f * fmaf((float)cx, us, pxx);
                 const float B = cy == 0 ? 1.f - pyy : 0.5f * fmaf((float)cy, vs, pyy);
                 const float ax = cx == 0 ? -1.f : 0.5f, ay = cy == 0 ? -1.f : 0.5f;
@@ -126,7 +127,7 @@ __device__ __forceinline__ void node_update(const T *__restrict__ in, T *__restr
     stf(out + p.fstride + k, uxn);
     stf(out + 2 * p.fstride + k, uyn);
     if (Q == 19) stf(out + 3 * p.fstride + k, jz / rn);
-    if (SC) stf(out + (Q == 19 ? 4 : 3) * p.fstride + k, fmaf(p.at, ldf(Tin + k), ts));
+    if (SC) stf(out + (Q == 19 ? 4 : 3) * p.fstride + k, fmaf(p.at, ldx<RO>(Tin + k), ts));
     if (BULK) stf(out + 3 * p.fstride + k, trs / rna - fmaf(uxn, uxn, uyn * uyn));
 }
 

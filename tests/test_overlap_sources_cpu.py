@@ -1,7 +1,9 @@
 """Kernels that overlap the grid before them (griddepcontrol.wait, programmatic stream
 serialization) must not read device memory through the read-only path: that path is defined only
 for data nobody writes while the kernel is alive, and such a kernel is alive while the grid before
-it still writes the state. Read from the sources, since a stale value cannot be provoked at will."""
+it still writes the state. Nor must kernels that run many steps in one launch, whose CTAs read what
+others wrote before a barrier. Read from the sources, since a stale value cannot be provoked at
+will."""
 import os
 import re
 
@@ -51,3 +53,18 @@ def test_no_read_only_loads(name):
     2D-tile kernels too, which overlap nothing; its march is that of rows2.cuh)."""
     text = source(name)
     assert "__ldg" not in text and not re.search(r"\bldf\s*\(", text)
+
+
+def test_persistent_kernels_read_with_ordinary_loads():
+    """Their updates are the single-step kernels' with RO (read-only) off; the march past L1."""
+    bodies = {k: (p, b) for k, p, b in kernels(source("kernels_batch.cu"))}
+    want = {"k_batch_persistent": "tile_update<Q, false>(", "k_batch_tiles_persistent": "tile2_update<TW, TH, false>(",
+            "k_batch_rows_persistent": "rows2_update<NS, T, true>("}
+    assert set(want) == {k for k in bodies if "grid_barrier" in bodies[k][1]}
+    for k, call in want.items():
+        params, body = bodies[k]
+        assert call in body and "__restrict__" not in params
+    for name in ("node_update.cuh", "kernels_batch.cu"):  # the state only through ldx<RO>
+        text = source(name)
+        assert not re.search(r"\bldf\s*\(", text)
+        assert all("field" in m for m in re.findall(r"__ldg\(([^)]*)\)", text))
