@@ -120,7 +120,8 @@ enum {
                                      before lwacm_bind; single-domain contexts only */
     LWACM_OPT_BATCH_TILE = 13,    /* how domains are cut into CTA tiles. Batched contexts:
                                      0 (default) = D2Q9: strips of 30 or 60 columns, each
-                                     updated by a warp that marches along y; D3Q19: runs
+                                     updated by a warp that marches along y; D3Q19 and
+                                     ensembles of narrow D2Q9 domains: runs
                                      of 256 consecutive nodes; 1..6 = 2D tiles of
                                      30x6, 30x14, 62x6, 30x30, 62x14, 126x6 nodes, D2Q9
                                      only (LWACM_E_UNSUPPORTED otherwise), with the link

@@ -1,15 +1,15 @@
 // Batched update of many independent periodic domains of different sizes and
 // viscosities, packed one after the other in the same field arrays.
 //
-// D2Q9 domains are cut into strips of columns and runs of rows, each updated by a warp
-// that marches along y (rows2.cuh), from a table of items that holds what a warp needs of
+// D2Q9 domains, but for ensembles of narrow ones, are cut into strips of columns and runs of
+// rows, each updated by a warp that marches along y (rows2.cuh), from a table of items that holds what a warp needs of
 // its domain. 256 domains of 32 to 512 nodes a side (seed 1 of the benchmark): 37 us a
 // step, 187 GLUPS, against 118 us with one thread a node gathering from global memory and
 // 65 us in 2D tiles; bound by the latency of the last wave of items and the part of the
 // state that L2 does not hold.
 //
-// D3Q19 domains are cut into tiles of 256 consecutive nodes (a tile never spans two
-// domains); a CTA walks the tile list with a grid stride, one node per thread,
+// D3Q19 domains and narrow D2Q9 ones are cut into tiles of 256 consecutive nodes (a tile never
+// spans two domains); a CTA walks the tile list with a grid stride, one node per thread,
 // and updates it with the per-node moment form of Eq. ACM2.0 (node_update.cuh)
 // using its domain's (nx, ny, nz, nu).
 //
@@ -581,11 +581,18 @@ cudaError_t persistent_t(void *b0, void *b1, const BatchParams &bp, long long ns
 }
 
 template <typename T>
-cudaError_t step_t(const void *in, void *out, const BatchParams &bp, cudaStream_t st) {
+cudaError_t step_t(int Q, const void *in, void *out, const BatchParams &bp, cudaStream_t st) {
     const long long cap = (long long)device_sms() * 8;
     const unsigned grid = (unsigned)(bp.ntiles < cap ? bp.ntiles : cap);
-    k_batch_step<19, T><<<grid, kTile, 0, st>>>((const T *)in, (T *)out, bp);
+    if (Q == 9)
+        k_batch_step<9, T><<<grid, kTile, 0, st>>>((const T *)in, (T *)out, bp);
+    else
+        k_batch_step<19, T><<<grid, kTile, 0, st>>>((const T *)in, (T *)out, bp);
     return cudaGetLastError();
+}
+template <typename T>
+cudaError_t runs_t(int Q, void *b0, void *b1, const BatchParams &bp, long long nsteps, int parity, cudaStream_t st) {
+    return Q == 9 ? persistent_t<9, T>(b0, b1, bp, nsteps, parity, st) : persistent_t<19, T>(b0, b1, bp, nsteps, parity, st);
 }
 
 }  // namespace
@@ -604,6 +611,20 @@ void batch_rows_cut(const BatchDomain *doms, int n, int *ns, int *rows) {
     const rows2::Cut c = rows2::cut_rows(w1, w2, 28LL * 152, 23LL * 152);
     *ns = c.ns;
     *rows = c.rows;
+}
+// A strip's row costs a warp the same whether the domain fills its 30 columns or one, a node of a run
+// 1 / 12 of it (one launch a step) or 1 / 15 (one launch for all); a launch of the strips' kernel,
+// which overlaps the one before, takes 0.8 us less. us a step, runs / strips, 1000 domains of 300
+// rows: 2 columns 12.8 / 63.1, 8 44.7 / 63.2, 10 52.7 / 63.3, 16 91 / 63; in one launch 8 columns 47 /
+// 77, 14 78 / 82; 300 domains of 8 x 64 4.2 / 4.9, of 10 x 64 5.2 / 4.9; 20 of 4 x 20 2.4 / 1.6; 4
+// of 300^2 with 60 of 3 x 300 6.9 / 6.7, with 200 11.2 / 16.3.
+bool batch_rows_pays(const BatchDomain *doms, int n, bool one_launch) {
+    long long nodes = 0, rows = 0;
+    for (int b = 0; b < n; ++b) {
+        nodes += doms[b].n;
+        rows += (long long)((doms[b].nx - 1) / rows2::kHalf + 1) * doms[b].ny;
+    }
+    return one_launch ? 15 * rows <= nodes + 6000 : 12 * rows <= nodes + 46000;
 }
 int batch_shapes() { return kNumShapes; }
 void batch_shape(int k, int *tw, int *th) {
@@ -641,11 +662,11 @@ cudaError_t launch_batch_step(int Q, int storage, const void *in, void *out, con
         if (!batch_shape_supported(Q, storage, bp.shape)) return cudaErrorInvalidValue;
         return tiles_storage(storage, in, out, nullptr, nullptr, bp, 1, 0, false, st);
     }
-    if (Q == 9) return rows_storage(storage, in, out, nullptr, nullptr, bp, 1, 0, false, st);
+    if (bp.rows2) return rows_storage(storage, in, out, nullptr, nullptr, bp, 1, 0, false, st);
     switch (storage) {
-        case STORE_F32: return step_t<float>(in, out, bp, st);
-        case STORE_BF16: return step_t<__nv_bfloat16>(in, out, bp, st);
-        case STORE_F16: return step_t<__half>(in, out, bp, st);
+        case STORE_F32: return step_t<float>(Q, in, out, bp, st);
+        case STORE_BF16: return step_t<__nv_bfloat16>(Q, in, out, bp, st);
+        case STORE_F16: return step_t<__half>(Q, in, out, bp, st);
     }
     return cudaErrorInvalidValue;
 }
@@ -658,11 +679,11 @@ cudaError_t launch_batch_persistent(int Q, int storage, void *buf0, void *buf1, 
         if (!batch_shape_supported(Q, storage, bp.shape)) return cudaErrorInvalidValue;
         return tiles_storage(storage, nullptr, nullptr, buf0, buf1, bp, nsteps, parity, true, st);
     }
-    if (Q == 9) return rows_storage(storage, nullptr, nullptr, buf0, buf1, bp, nsteps, parity, true, st);
+    if (bp.rows2) return rows_storage(storage, nullptr, nullptr, buf0, buf1, bp, nsteps, parity, true, st);
     switch (storage) {
-        case STORE_F32: return persistent_t<19, float>(buf0, buf1, bp, nsteps, parity, st);
-        case STORE_BF16: return persistent_t<19, __nv_bfloat16>(buf0, buf1, bp, nsteps, parity, st);
-        case STORE_F16: return persistent_t<19, __half>(buf0, buf1, bp, nsteps, parity, st);
+        case STORE_F32: return runs_t<float>(Q, buf0, buf1, bp, nsteps, parity, st);
+        case STORE_BF16: return runs_t<__nv_bfloat16>(Q, buf0, buf1, bp, nsteps, parity, st);
+        case STORE_F16: return runs_t<__half>(Q, buf0, buf1, bp, nsteps, parity, st);
     }
     return cudaErrorInvalidValue;
 }

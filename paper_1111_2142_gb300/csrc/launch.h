@@ -72,13 +72,15 @@ struct BatchRows {
 // strips per warp (1 or 2) and rows per item for an ensemble
 void batch_rows_cut(const BatchDomain *doms, int n, int *ns, int *rows);
 int batch_rows_strip();  // columns of a strip
+// whether the strips are the faster ones for an ensemble, not 1D tiles (a launch a step or one for all)
+bool batch_rows_pays(const BatchDomain *doms, int n, bool one_launch);
 struct BatchParams {
     const BatchDomain *doms;
     const BatchTile *tiles;
     const BatchTile2 *tiles2;  // same storage as tiles, used when shape > 0
-    const BatchRows *rows2;    // same storage, used for D2Q9 and shape 0
+    const BatchRows *rows2;    // shape 0: strips marched along y (D2Q9; nullptr: 1D tiles)
     int ns;                    // strips per warp of rows2
-    int shape;                 // 0: rows2 (D2Q9) or 1D tiles of batch_tile() nodes; k > 0: 2D shape k
+    int shape;                 // 0: rows2 or 1D tiles of batch_tile() nodes; k > 0: 2D shape k
     long long ntiles;
     long long fstride;
     unsigned *bar_count;  // followed by the barrier generation word

@@ -78,8 +78,11 @@ struct lwacm_ctx {
     // batched domains (nbatch > 0): packed one after the other
     int nbatch = 0;
     std::vector<BatchDomain> doms;
-    std::vector<BatchTile> tiles;    // 1D tiles (D3Q19, shape 0)
-    std::vector<BatchRows> rows2;    // strips and runs of rows (D2Q9, shape 0)
+    // shape 0: 1D tiles (D3Q19, narrow D2Q9 domains), strips and runs of rows (D2Q9), by launch form;
+    // an ensemble near the line between them has both tables, the tiles after the rows
+    std::vector<BatchTile> tiles;
+    std::vector<BatchRows> rows2;
+    bool rows_pay[2] = {false, false};
     int rows_ns = 1;                 // strips per warp of rows2
     std::vector<BatchTile2> tiles2;  // 2D tiles of the current shape (shape > 0)
     int batch_shape = 0;
@@ -218,7 +221,7 @@ bool choose_kernel(lwacm_ctx *c) {
             {"batch_persistent", "batch_tiles30x6_persistent", "batch_tiles30x14_persistent",
              "batch_tiles62x6_persistent", "batch_tiles30x30_persistent", "batch_tiles62x14_persistent",
              "batch_tiles126x6_persistent", "batch_rows_persistent"}};
-        c->kname = names[c->batch_mode ? 1 : 0][c->batch_shape == 0 && c->Q == 9 ? 7 : c->batch_shape];
+        c->kname = names[c->batch_mode ? 1 : 0][c->batch_shape == 0 && c->rows_pay[c->batch_mode] ? 7 : c->batch_shape];
         return c->kernel_opt == 0 || c->kernel_opt == 1;
     }
     const StepParams p = params(c);
@@ -315,14 +318,14 @@ lwacm_status upload_tiles(lwacm_ctx *c) {
         CK(c, cudaMemcpyAsync(c->ws + c->off_tiles, c->tiles2.data(), sizeof(BatchTile2) * c->tiles2.size(),
                               cudaMemcpyHostToDevice, c->stream),
            "tile table");
-    } else if (c->Q == 9) {
-        CK(c, cudaMemcpyAsync(c->ws + c->off_tiles, c->rows2.data(), sizeof(BatchRows) * c->rows2.size(),
-                              cudaMemcpyHostToDevice, c->stream),
-           "tile table");
     } else {
-        CK(c, cudaMemcpyAsync(c->ws + c->off_tiles, c->tiles.data(), sizeof(BatchTile) * c->tiles.size(),
-                              cudaMemcpyHostToDevice, c->stream),
-           "tile table");
+        const size_t rb = sizeof(BatchRows) * c->rows2.size(), tb = sizeof(BatchTile) * c->tiles.size();
+        if (rb)
+            CK(c, cudaMemcpyAsync(c->ws + c->off_tiles, c->rows2.data(), rb, cudaMemcpyHostToDevice, c->stream),
+               "tile table");
+        if (tb)
+            CK(c, cudaMemcpyAsync(c->ws + c->off_tiles + rb, c->tiles.data(), tb, cudaMemcpyHostToDevice, c->stream),
+               "tile table");
     }
     CK(c, cudaStreamSynchronize(c->stream), "sync");
     return LWACM_OK;
@@ -331,12 +334,13 @@ lwacm_status upload_tiles(lwacm_ctx *c) {
 BatchParams batch_params(lwacm_ctx *c) {
     BatchParams bp;
     bp.doms = (const BatchDomain *)(c->ws + c->off_doms);
-    bp.tiles = (const BatchTile *)(c->ws + c->off_tiles);
+    const bool rows = c->rows_pay[c->batch_mode];
+    bp.tiles = (const BatchTile *)(c->ws + c->off_tiles + sizeof(BatchRows) * c->rows2.size());
     bp.tiles2 = (const BatchTile2 *)(c->ws + c->off_tiles);
-    bp.rows2 = (const BatchRows *)(c->ws + c->off_tiles);
+    bp.rows2 = rows ? (const BatchRows *)(c->ws + c->off_tiles) : nullptr;
     bp.ns = c->rows_ns;
     bp.shape = c->batch_shape;
-    bp.ntiles = (long long)(c->batch_shape > 0 ? c->tiles2.size() : (c->Q == 9 ? c->rows2.size() : c->tiles.size()));
+    bp.ntiles = (long long)(c->batch_shape > 0 ? c->tiles2.size() : (rows ? c->rows2.size() : c->tiles.size()));
     bp.fstride = c->Nal;
     bp.bar_count = (unsigned *)(c->ws + c->off_bar);
     bp.bar_gen = bp.bar_count + 1;
@@ -640,24 +644,26 @@ lwacm_status lwacm_batch_create(int lattice, int n, const int *nx, const int *ny
             d.n = (long long)nx[b] * ny[b] * z;
             d.s = (float)(18.0 * nu[b]);  // Eq. ACM2.0nu: s = 18 nu, a = 1 - 6 nu
             d.a = (float)(1.0 - 6.0 * nu[b]);
-            for (long long t = 0; lattice == LWACM_D3Q19 && t < d.n; t += tile) {
+            off += d.n;
+        }
+        for (int m = 0; m < 2; ++m)
+            c->rows_pay[m] = lattice == LWACM_D2Q9 && batch_rows_pays(c->doms.data(), n, m == 1);
+        for (int b = 0; b < n && !(c->rows_pay[0] && c->rows_pay[1]); ++b)
+            for (long long t = 0; t < c->doms[b].n; t += tile) {
                 BatchTile bt;
                 bt.dom = b;
                 bt.pad = 0;
-                bt.start = off + t;
+                bt.start = c->doms[b].off + t;
                 c->tiles.push_back(bt);
             }
-            off += d.n;
-        }
     } catch (...) {
         delete c;
         return LWACM_E_NOMEM;
     }
     try {
-        c->tiles_cap = sizeof(BatchTile) * c->tiles.size();
+        if (c->rows_pay[0] || c->rows_pay[1]) build_rows2(c);
+        c->tiles_cap = sizeof(BatchRows) * c->rows2.size() + sizeof(BatchTile) * c->tiles.size();
         if (lattice == LWACM_D2Q9) {
-            build_rows2(c);
-            c->tiles_cap = sizeof(BatchRows) * c->rows2.size();
             std::vector<BatchTile2> t2;
             for (int k = 1; k < batch_shapes(); ++k) {
                 build_tiles2(c, k, t2);
