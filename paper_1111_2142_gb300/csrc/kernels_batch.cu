@@ -612,19 +612,19 @@ void batch_rows_cut(const BatchDomain *doms, int n, int *ns, int *rows) {
     *ns = c.ns;
     *rows = c.rows;
 }
-// A strip's row costs a warp the same whether the domain fills its 30 columns or one, a node of a run
-// 1 / 12 of it (one launch a step) or 1 / 15 (one launch for all); a launch of the strips' kernel,
-// which overlaps the one before, takes 0.8 us less. us a step, runs / strips, 1000 domains of 300
-// rows: 2 columns 12.8 / 63.1, 8 44.7 / 63.2, 10 52.7 / 63.3, 16 91 / 63; in one launch 8 columns 47 /
-// 77, 14 78 / 82; 300 domains of 8 x 64 4.2 / 4.9, of 10 x 64 5.2 / 4.9; 20 of 4 x 20 2.4 / 1.6; 4
-// of 300^2 with 60 of 3 x 300 6.9 / 6.7, with 200 11.2 / 16.3.
-bool batch_rows_pays(const BatchDomain *doms, int n, bool one_launch) {
+// A strip's row costs a warp the same whether the domain fills its 30 columns or one, a node of a
+// run 1 / 12 of it; a launch of the strips' kernel, which overlaps the one before, takes 0.8 us less.
+// us a step, runs / strips, 1000 domains of 300 rows: 2 columns 12.8 / 63.1, 8 44.7 / 63.2, 10 52.7 /
+// 63.3, 16 91 / 63; 300 domains of 8 x 64 4.2 / 4.9, of 10 x 64 5.2 / 4.9; 20 of 4 x 20 2.4 / 1.6; 4
+// of 300^2 with 60 of 3 x 300 6.9 / 6.7, with 200 11.2 / 16.3. Both launch forms take the same kernel
+// and so give the same fields (in one launch the line lies some nodes higher).
+bool batch_rows_pays(const BatchDomain *doms, int n) {
     long long nodes = 0, rows = 0;
     for (int b = 0; b < n; ++b) {
         nodes += doms[b].n;
         rows += (long long)((doms[b].nx - 1) / rows2::kHalf + 1) * doms[b].ny;
     }
-    return one_launch ? 15 * rows <= nodes + 6000 : 12 * rows <= nodes + 46000;
+    return 12 * rows <= nodes + 46000;
 }
 int batch_shapes() { return kNumShapes; }
 void batch_shape(int k, int *tw, int *th) {

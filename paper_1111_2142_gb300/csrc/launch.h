@@ -72,8 +72,8 @@ struct BatchRows {
 // strips per warp (1 or 2) and rows per item for an ensemble
 void batch_rows_cut(const BatchDomain *doms, int n, int *ns, int *rows);
 int batch_rows_strip();  // columns of a strip
-// whether the strips are the faster ones for an ensemble, not 1D tiles (a launch a step or one for all)
-bool batch_rows_pays(const BatchDomain *doms, int n, bool one_launch);
+// whether the strips are the faster ones for an ensemble, not 1D tiles
+bool batch_rows_pays(const BatchDomain *doms, int n);
 struct BatchParams {
     const BatchDomain *doms;
     const BatchTile *tiles;

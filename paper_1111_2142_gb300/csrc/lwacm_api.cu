@@ -78,11 +78,10 @@ struct lwacm_ctx {
     // batched domains (nbatch > 0): packed one after the other
     int nbatch = 0;
     std::vector<BatchDomain> doms;
-    // shape 0: 1D tiles (D3Q19, narrow D2Q9 domains), strips and runs of rows (D2Q9), by launch form;
-    // an ensemble near the line between them has both tables, the tiles after the rows
-    std::vector<BatchTile> tiles;
+    // shape 0: strips and runs of rows (D2Q9) or 1D tiles (D3Q19, narrow D2Q9 domains; rows2 is empty),
+    // the same in both launch forms, which give the same fields bit for bit
     std::vector<BatchRows> rows2;
-    bool rows_pay[2] = {false, false};
+    std::vector<BatchTile> tiles;
     int rows_ns = 1;                 // strips per warp of rows2
     std::vector<BatchTile2> tiles2;  // 2D tiles of the current shape (shape > 0)
     int batch_shape = 0;
@@ -221,7 +220,7 @@ bool choose_kernel(lwacm_ctx *c) {
             {"batch_persistent", "batch_tiles30x6_persistent", "batch_tiles30x14_persistent",
              "batch_tiles62x6_persistent", "batch_tiles30x30_persistent", "batch_tiles62x14_persistent",
              "batch_tiles126x6_persistent", "batch_rows_persistent"}};
-        c->kname = names[c->batch_mode ? 1 : 0][c->batch_shape == 0 && c->rows_pay[c->batch_mode] ? 7 : c->batch_shape];
+        c->kname = names[c->batch_mode ? 1 : 0][c->batch_shape == 0 && !c->rows2.empty() ? 7 : c->batch_shape];
         return c->kernel_opt == 0 || c->kernel_opt == 1;
     }
     const StepParams p = params(c);
@@ -318,14 +317,14 @@ lwacm_status upload_tiles(lwacm_ctx *c) {
         CK(c, cudaMemcpyAsync(c->ws + c->off_tiles, c->tiles2.data(), sizeof(BatchTile2) * c->tiles2.size(),
                               cudaMemcpyHostToDevice, c->stream),
            "tile table");
+    } else if (!c->rows2.empty()) {
+        CK(c, cudaMemcpyAsync(c->ws + c->off_tiles, c->rows2.data(), sizeof(BatchRows) * c->rows2.size(),
+                              cudaMemcpyHostToDevice, c->stream),
+           "tile table");
     } else {
-        const size_t rb = sizeof(BatchRows) * c->rows2.size(), tb = sizeof(BatchTile) * c->tiles.size();
-        if (rb)
-            CK(c, cudaMemcpyAsync(c->ws + c->off_tiles, c->rows2.data(), rb, cudaMemcpyHostToDevice, c->stream),
-               "tile table");
-        if (tb)
-            CK(c, cudaMemcpyAsync(c->ws + c->off_tiles + rb, c->tiles.data(), tb, cudaMemcpyHostToDevice, c->stream),
-               "tile table");
+        CK(c, cudaMemcpyAsync(c->ws + c->off_tiles, c->tiles.data(), sizeof(BatchTile) * c->tiles.size(),
+                              cudaMemcpyHostToDevice, c->stream),
+           "tile table");
     }
     CK(c, cudaStreamSynchronize(c->stream), "sync");
     return LWACM_OK;
@@ -334,8 +333,8 @@ lwacm_status upload_tiles(lwacm_ctx *c) {
 BatchParams batch_params(lwacm_ctx *c) {
     BatchParams bp;
     bp.doms = (const BatchDomain *)(c->ws + c->off_doms);
-    const bool rows = c->rows_pay[c->batch_mode];
-    bp.tiles = (const BatchTile *)(c->ws + c->off_tiles + sizeof(BatchRows) * c->rows2.size());
+    const bool rows = !c->rows2.empty();
+    bp.tiles = (const BatchTile *)(c->ws + c->off_tiles);
     bp.tiles2 = (const BatchTile2 *)(c->ws + c->off_tiles);
     bp.rows2 = rows ? (const BatchRows *)(c->ws + c->off_tiles) : nullptr;
     bp.ns = c->rows_ns;
@@ -646,9 +645,9 @@ lwacm_status lwacm_batch_create(int lattice, int n, const int *nx, const int *ny
             d.a = (float)(1.0 - 6.0 * nu[b]);
             off += d.n;
         }
-        for (int m = 0; m < 2; ++m)
-            c->rows_pay[m] = lattice == LWACM_D2Q9 && batch_rows_pays(c->doms.data(), n, m == 1);
-        for (int b = 0; b < n && !(c->rows_pay[0] && c->rows_pay[1]); ++b)
+        const bool rows = lattice == LWACM_D2Q9 && batch_rows_pays(c->doms.data(), n);
+        if (rows) build_rows2(c);
+        for (int b = 0; b < n && !rows; ++b)
             for (long long t = 0; t < c->doms[b].n; t += tile) {
                 BatchTile bt;
                 bt.dom = b;
@@ -661,8 +660,7 @@ lwacm_status lwacm_batch_create(int lattice, int n, const int *nx, const int *ny
         return LWACM_E_NOMEM;
     }
     try {
-        if (c->rows_pay[0] || c->rows_pay[1]) build_rows2(c);
-        c->tiles_cap = sizeof(BatchRows) * c->rows2.size() + sizeof(BatchTile) * c->tiles.size();
+        c->tiles_cap = sizeof(BatchRows) * c->rows2.size() + sizeof(BatchTile) * c->tiles.size();  // one is empty
         if (lattice == LWACM_D2Q9) {
             std::vector<BatchTile2> t2;
             for (int k = 1; k < batch_shapes(); ++k) {
