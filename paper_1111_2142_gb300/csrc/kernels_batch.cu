@@ -613,18 +613,19 @@ void batch_rows_cut(const BatchDomain *doms, int n, int *ns, int *rows) {
     *rows = c.rows;
 }
 // A strip's row costs a warp the same whether the domain fills its 30 columns or one, a node of a
-// run 1 / 12 of it; a launch of the strips' kernel, which overlaps the one before, takes 0.8 us less.
-// us a step, runs / strips, 1000 domains of 300 rows: 2 columns 12.8 / 63.1, 8 44.7 / 63.2, 10 52.7 /
-// 63.3, 16 91 / 63; 300 domains of 8 x 64 4.2 / 4.9, of 10 x 64 5.2 / 4.9; 20 of 4 x 20 2.4 / 1.6; 4
-// of 300^2 with 60 of 3 x 300 6.9 / 6.7, with 200 11.2 / 16.3. Both launch forms take the same kernel
-// and so give the same fields (in one launch the line lies some nodes higher).
+// run 1 / 9 of it; a launch of the strips' kernel, which overlaps the one before, takes 0.8 us less.
+// us a step, runs / strips, 1000 domains of 300 rows: 2 columns 12.8 / 44.8, 6 36.7 / 44.8, 8 44.7 /
+// 44.9, 10 52.7 / 46; 300 domains of 8 x 64 4.2 / 4.9, of 10 x 64 5.2 / 4.9; 20 of 4 x 20 2.4 / 1.6; 4 of
+// 300^2 with 60 of 3 x 300 6.9 / 6.7, with 200 11.2 / 13.3. Both launch forms take the same kernel and
+// so give the same fields; in one launch for all steps the line lies some nodes higher (20 domains of
+// 10 x 200 4.6 / 5.2, 1000 of 10 x 300 57 / 57).
 bool batch_rows_pays(const BatchDomain *doms, int n) {
     long long nodes = 0, rows = 0;
     for (int b = 0; b < n; ++b) {
         nodes += doms[b].n;
         rows += (long long)((doms[b].nx - 1) / rows2::kHalf + 1) * doms[b].ny;
     }
-    return 12 * rows <= nodes + 46000;
+    return 10 * rows <= nodes + 10000;
 }
 int batch_shapes() { return kNumShapes; }
 void batch_shape(int k, int *tw, int *th) {

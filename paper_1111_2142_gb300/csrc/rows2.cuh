@@ -50,7 +50,10 @@ inline int cta_warps(int nx) {
 // to 8 (1024^2: 6 rows 6.5, 4 rows 7.3; the cavity 8 rows 7.4, 6 rows 8.9). Larger domains
 // take 8 to 16 rows, whichever wastes least of the last wave (2048^2: 10 rows 18.1, 16 rows
 // 19.5), 16 where there are more than 4 waves (4096^2: 70.8, 64 rows 84) and 32 where there
-// are more than 9 (8192^2: 262, 24 rows 266).
+// are more than 9 (8192^2: 262, 24 rows 266). Two strips a warp only where they are mostly
+// there: in domains of up to 30 columns the second one is empty (30 x 65536 nodes, one strip /
+// two: 11.3 / 15.3, bulk viscosity 18.8 / 30.3, the 2D tiles 25.7; 1000 domains of 20 x 300
+// 47.6 / 67.4).
 struct Cut {
     int ns, rows;
 };
@@ -59,15 +62,17 @@ inline Cut cut_rows(long long w1, long long w2, long long room1, long long room2
     const long long once1 = (w1 - 1) / room1 + 1, once2 = (w2 - 1) / room2 + 1;
     Cut c{1, (int)once1};
     if (once1 > 5) {
-        c.ns = 2;
+        const bool two = 4 * w2 <= 3 * w1;
+        const long long w = two ? w2 : w1, room = two ? room2 : room1, once = two ? once2 : once1;
+        c.ns = two ? 2 : 1;
         c.rows = 16;
-        if (once2 <= 8)
-            c.rows = (int)once2;
-        else if (w2 > 9 * 16 * room2)
+        if (once <= 8)
+            c.rows = (int)once;
+        else if (w > 9 * 16 * room)
             c.rows = 32;
-        else if (w2 <= 4 * 16 * room2)
+        else if (w <= 4 * 16 * room)
             for (int h = 16, best = 1 << 30; h >= 8; --h) {
-                const int cost = (int)((w2 / h + room2) / room2) * (2 * h + 3);
+                const int cost = (int)((w / h + room) / room) * (2 * h + 3);
                 if (cost < best) best = cost, c.rows = h;
             }
     }

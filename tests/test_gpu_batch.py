@@ -189,10 +189,10 @@ def test_ensemble_256(lw):
     sim.close()
 
 
-# ensembles each side of the line between strips and 1D runs (12 nodes a strip's row, small ones
+# ensembles each side of the line between strips and 1D runs (10 nodes a strip's row, small ones
 # on strips): narrow and wide domains, mixtures
 @pytest.mark.parametrize("storage", [0, 1])
-@pytest.mark.parametrize("dims,rows", [([(1, 6000), (2, 2300), (3, 7)], False), ([(11, 4000)] * 12, False), ([(12, 1950), (13, 1721)], True),
+@pytest.mark.parametrize("dims,rows", [([(1, 3000), (2, 2300), (3, 7)], False), ([(7, 4000)] * 6, False), ([(9, 1950), (8, 1721)], True),
                                        ([(22, 64), (31, 9)], True), ([(1, 40), (2, 90), (3, 33)], True),
                                        ([(60, 41), (2, 90), (90, 33)], True), ([(60, 200)] + [(3, 800)] * 9, False)])
 def test_narrow_ensembles(lw, dims, rows, storage):

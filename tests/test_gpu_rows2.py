@@ -124,3 +124,18 @@ def test_ensemble_strips_equal_single_domains(lw, storage, scale):
             for x, y in zip(g, one.get_fields()):
                 assert np.array_equal(x, y), (mode, w, h)
             one.close()
+
+
+# more rows than the GPU holds warps at once, five and more rows an item: up to 30 columns on one
+# strip a warp, up to 60 on two; both edges
+@pytest.mark.parametrize("shape", [(30011, 1), (30011, 29), (26003, 30), (30011, 31), (25013, 60), (25013, 61)])
+def test_tall_narrow_domains(lw, shape):
+    """The plain scheme and a cavity against the oracle, the bulk variant against the tile kernel."""
+    f = inputs.smooth_random(shape, seed=26, u_amp=0.05, d_amp=0.01)
+    within(run(lw, shape, f, 3), oracle.step(9, *f, nu=0.02, nsteps=3))
+    if shape[1] > 1:
+        within(run(lw, shape, f, 3, 1, lid=(0.05, 0.01)),
+               oracle.step(9, *f, nu=0.02, bc=1, nsteps=3, lid=(0.05, 0.01, 0.0)))
+    a, b = (run(lw, shape, f, 3, tile=t, bulk_gamma=0.4) for t in (0, 2))
+    for x, y in zip(a, b):
+        assert np.array_equal(x, y)
