@@ -550,6 +550,15 @@ cudaError_t rows_t(const void *in, void *out, void *b0, void *b1, const BatchPar
     return cudaLaunchCooperativeKernel((const void *)k_batch_rows_persistent<NS, T>, dim3((unsigned)grid), dim3(kTile),
                                        args, 0, st);
 }
+// warps of the kernel that the GPU holds (-1 when it cannot be determined)
+template <int NS, typename T>
+int rows_room(bool one_launch) {
+    static DevSlots cap[2];
+    const int w = one_launch ? kTile / 32 : rows_warps(NS);
+    const int g = one_launch ? max_grid(k_batch_rows_persistent<NS, T>, 32 * w, cap[1])
+                             : max_grid(k_batch_rows<NS, T>, 32 * w, cap[0]);
+    return g < 1 ? -1 : g * w;
+}
 cudaError_t rows_storage(int storage, const void *in, void *out, void *b0, void *b1, const BatchParams &bp,
                          long long nsteps, int parity, bool persistent, cudaStream_t st) {
     switch (storage) {
@@ -599,16 +608,30 @@ cudaError_t runs_t(int Q, void *b0, void *b1, const BatchParams &bp, long long n
 
 int batch_tile() { return kTile; }
 int batch_rows_strip() { return rows2::kHalf; }
-// the cut of one domain (rows2.cuh) over the whole ensemble's strips, for the warps the GPU
-// holds (28 a SM of the one-strip form, 23 of the other). 256 domains of 32 to 512 nodes a
-// side: 17 rows 37.7 us a step, 4 rows 46.3, 64 rows 45.2, one strip a warp 42.4 at best.
-void batch_rows_cut(const BatchDomain *doms, int n, int *ns, int *rows) {
+// The cut of one domain (rows2.cuh) over the whole ensemble's strips, for the warps the GPU holds of
+// the kernel that runs (28 or 32 a SM of the one-strip form with a launch a step, 23 of the other,
+// 24 and 16 in one launch for all; `device`: asked of the current one, else those of a GB300). 256
+// domains of 32 to 512 nodes a side: 17 rows 37.7 us a step, 4 rows 46.3, 64 rows 45.2, one strip a
+// warp 42.4 at best. The one-launch form cut for its own room, in place of the other form's: 20
+// domains of 10 x 200 4.1 us a step against 5.7, 300 of 10 x 64 7.2 against 9.3, 100 of 300^2 54.9
+// against 63.1.
+void batch_rows_cut(const BatchDomain *doms, int n, int storage, bool one_launch, bool device, int *ns, int *rows) {
     long long w1 = 0, w2 = 0;
     for (int b = 0; b < n; ++b) {
         w1 += (long long)((doms[b].nx - 1) / rows2::kHalf + 1) * doms[b].ny;
         w2 += (long long)((doms[b].nx - 1) / (2 * rows2::kHalf) + 1) * doms[b].ny;
     }
-    const rows2::Cut c = rows2::cut_rows(w1, w2, 28LL * 152, 23LL * 152);
+    long long r1 = (one_launch ? 24 : 28) * 152, r2 = (one_launch ? 16 : 23) * 152;
+    if (device) {
+        const int d1 = storage == STORE_F32    ? rows_room<1, float>(one_launch)
+                       : storage == STORE_BF16 ? rows_room<1, __nv_bfloat16>(one_launch)
+                                               : rows_room<1, __half>(one_launch);
+        const int d2 = storage == STORE_F32    ? rows_room<2, float>(one_launch)
+                       : storage == STORE_BF16 ? rows_room<2, __nv_bfloat16>(one_launch)
+                                               : rows_room<2, __half>(one_launch);
+        if (d1 > 0 && d2 > 0) r1 = d1, r2 = d2;
+    }
+    const rows2::Cut c = rows2::cut_rows(w1, w2, r1, r2);
     *ns = c.ns;
     *rows = c.rows;
 }
@@ -617,8 +640,7 @@ void batch_rows_cut(const BatchDomain *doms, int n, int *ns, int *rows) {
 // us a step, runs / strips, 1000 domains of 300 rows: 2 columns 12.8 / 44.8, 6 36.7 / 44.8, 8 44.7 /
 // 44.9, 10 52.7 / 46; 300 domains of 8 x 64 4.2 / 4.9, of 10 x 64 5.2 / 4.9; 20 of 4 x 20 2.4 / 1.6; 4 of
 // 300^2 with 60 of 3 x 300 6.9 / 6.7, with 200 11.2 / 13.3. Both launch forms take the same kernel and
-// so give the same fields; in one launch for all steps the line lies some nodes higher (20 domains of
-// 10 x 200 4.6 / 5.2, 1000 of 10 x 300 57 / 57).
+// so give the same fields (in one launch 20 domains of 10 x 200 4.6 / 4.1, 1000 of 10 x 300 57 / 57).
 bool batch_rows_pays(const BatchDomain *doms, int n) {
     long long nodes = 0, rows = 0;
     for (int b = 0; b < n; ++b) {

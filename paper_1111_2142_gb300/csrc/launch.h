@@ -69,8 +69,8 @@ struct BatchRows {
     float s, a;
     int pad[3];
 };
-// strips per warp (1 or 2) and rows per item for an ensemble
-void batch_rows_cut(const BatchDomain *doms, int n, int *ns, int *rows);
+// strips per warp (1 or 2) and rows per item for an ensemble, by launch form; device: for the current one
+void batch_rows_cut(const BatchDomain *doms, int n, int storage, bool one_launch, bool device, int *ns, int *rows);
 int batch_rows_strip();  // columns of a strip
 // whether the strips are the faster ones for an ensemble, not 1D tiles
 bool batch_rows_pays(const BatchDomain *doms, int n);

@@ -288,10 +288,11 @@ void build_tiles2(const lwacm_ctx *c, int k, std::vector<BatchTile2> &out) {
             for (int x = 0; x < c->doms[b].nx; x += tw) out.push_back(BatchTile2{b, x, y, 0});
 }
 
-// strips and runs of rows over every domain (D2Q9, shape 0)
-void build_rows2(lwacm_ctx *c) {
+// strips and runs of rows over every domain (D2Q9, shape 0) for a launch form; device: cut for the
+// current device
+void build_rows2(lwacm_ctx *c, int mode, bool device) {
     int rows = 1;
-    batch_rows_cut(c->doms.data(), c->nbatch, &c->rows_ns, &rows);
+    batch_rows_cut(c->doms.data(), c->nbatch, c->storage, mode == 1, device, &c->rows_ns, &rows);
     const int width = c->rows_ns * batch_rows_strip();
     c->rows2.clear();
     for (const BatchDomain &d : c->doms)
@@ -310,8 +311,16 @@ void build_rows2(lwacm_ctx *c) {
             }
 }
 
-// upload the tile table of the current shape (host tables are pageable: synchronise)
+// upload the tile table of the current shape and launch form (host tables are pageable: synchronise)
 lwacm_status upload_tiles(lwacm_ctx *c) {
+    if (!c->rows2.empty()) {
+        try {  // cut for this device, or as the workspace was sized
+            build_rows2(c, c->batch_mode, true);
+            if (sizeof(BatchRows) * c->rows2.size() > c->tiles_cap) build_rows2(c, c->batch_mode, false);
+        } catch (...) {
+            return fail(c, LWACM_E_NOMEM, "table of strips");
+        }
+    }
     if (c->batch_shape > 0) {
         build_tiles2(c, c->batch_shape, c->tiles2);
         CK(c, cudaMemcpyAsync(c->ws + c->off_tiles, c->tiles2.data(), sizeof(BatchTile2) * c->tiles2.size(),
@@ -646,7 +655,10 @@ lwacm_status lwacm_batch_create(int lattice, int n, const int *nx, const int *ny
             off += d.n;
         }
         const bool rows = lattice == LWACM_D2Q9 && batch_rows_pays(c->doms.data(), n);
-        if (rows) build_rows2(c);
+        for (int m = 1; rows && m >= 0; --m) {
+            build_rows2(c, m, false);
+            c->tiles_cap = std::max(c->tiles_cap, sizeof(BatchRows) * c->rows2.size());
+        }
         for (int b = 0; b < n && !rows; ++b)
             for (long long t = 0; t < c->doms[b].n; t += tile) {
                 BatchTile bt;
@@ -660,7 +672,7 @@ lwacm_status lwacm_batch_create(int lattice, int n, const int *nx, const int *ny
         return LWACM_E_NOMEM;
     }
     try {
-        c->tiles_cap = sizeof(BatchRows) * c->rows2.size() + sizeof(BatchTile) * c->tiles.size();  // one is empty
+        c->tiles_cap = std::max(c->tiles_cap, sizeof(BatchTile) * c->tiles.size());
         if (lattice == LWACM_D2Q9) {
             std::vector<BatchTile2> t2;
             for (int k = 1; k < batch_shapes(); ++k) {
@@ -745,7 +757,12 @@ lwacm_status lwacm_set_option(lwacm_ctx *c, int key, double v) {
             const int m = (int)v;
             if (m != 0 && m != 1) return fail(c, LWACM_E_ARG, "batch mode must be 0 or 1");
             if (!c->nbatch) return fail(c, LWACM_E_STATE, "not a batched context");
+            const bool other = m != c->batch_mode;
             c->batch_mode = m;
+            if (other && c->bound && !c->rows2.empty() && c->batch_shape == 0) {
+                const lwacm_status ts = upload_tiles(c);
+                if (ts != LWACM_OK) return ts;
+            }
             break;
         }
         case LWACM_OPT_SCALAR_ALPHA: {
