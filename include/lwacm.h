@@ -335,11 +335,15 @@ lwacm_status lwacm_diagnostics(lwacm_ctx *ctx, double out[8]);
 lwacm_status lwacm_adjoint_workspace_bytes(const lwacm_ctx *ctx, long long T, int stride,
                                            size_t *bytes);
 
-/* Advance the current state by T steps (as lwacm_step) while keeping a checkpoint
+/* Advance the current state by T steps while keeping a checkpoint
  * every S steps in the caller's device workspace (256-byte aligned, >=
  * lwacm_adjoint_workspace_bytes). The context then holds the state after T steps
  * and remembers the run for lwacm_backward; the workspace must stay valid until
- * then. */
+ * then. The steps are those of lwacm_step but for the order of their additions where
+ * lwacm_step runs marching warps: a recorded run takes the half-row kernel, the 2D
+ * tiles or the gather, so that dL/dnu, a sum that may cancel, does not depend on which
+ * kernel is the fastest. Fields equal bit for bit come from lwacm_step with
+ * LWACM_OPT_KERNEL 5 (D3Q19 shapes it takes) or LWACM_OPT_BATCH_TILE 2 (D2Q9). */
 lwacm_status lwacm_forward_record(lwacm_ctx *ctx, long long T, int stride, void *dev_workspace,
                                   size_t bytes);
 

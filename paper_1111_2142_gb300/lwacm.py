@@ -531,7 +531,8 @@ _LwacmRun = None
 
 def run(sim, T, nu, *fields, stride=0):
     """Differentiable T-step run: returns the fields after T steps; gradients flow
-    to `fields` and to the 0-d tensor `nu` (which must equal the sim's viscosity)."""
+    to `fields` and to the 0-d tensor `nu` (which must equal the sim's viscosity). The
+    fields are those of sim.step(T) to FP32 rounding (lwacm_forward_record)."""
     global _LwacmRun
     if _LwacmRun is None:
         _LwacmRun = _make_function()
