@@ -237,6 +237,10 @@ class Lwacm:
             self._hold = keep  # host memory must outlive the asynchronous copy
             self.sync()
             self._hold = None
+        else:
+            for a in keep:  # the copy runs on the library's stream
+                if a.is_cuda:
+                    a.record_stream(self.stream)
 
     def set_force_field(self, gx, gy, gz=None):
         """Per-node acceleration g(x) of Eq. force for the following steps (needs

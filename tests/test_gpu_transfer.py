@@ -117,3 +117,29 @@ def test_force_field_from_memory_of_another_device(lw):
         assert np.array_equal(x, y)
     assert float(np.max(np.abs(out[0][1]))) > 1e-5
     sim.close()
+
+
+@pytest.mark.parametrize("strided", [False, True])
+def test_fields_outlive_the_call_on_another_stream(lw, strided):
+    """Arrays that are dropped right after set_fields (or copies made of strided ones) are not handed
+    out again while the copy still waits on the context's own stream."""
+    import torch
+    n = 64
+    st = torch.cuda.Stream()
+    sim = lw.Lwacm(9, n, n, 1, 0.02, stream=st)
+    g = torch.Generator(device="cuda").manual_seed(84)
+    f = [torch.randn(n, n, generator=g, device="cuda") * 0.05 for _ in range(3)]
+    if strided:
+        f = [t.t() for t in f]
+    want = [t.cpu().numpy().astype(np.float64) for t in f]
+    torch.cuda.synchronize()
+    with torch.cuda.stream(st):
+        torch.cuda._sleep(50_000_000)  # some 30 ms during which the copy cannot start
+    sim.set_fields(*f)
+    del f
+    other = [torch.full((n, n), 7.0, device="cuda") for _ in range(6)]
+    torch.cuda.current_stream().synchronize()
+    for a, b in zip(want, sim.get_fields()):
+        assert np.array_equal(a, b)
+    assert all(float(t[0, 0]) == 7.0 for t in other)
+    sim.close()
