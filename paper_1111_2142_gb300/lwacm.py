@@ -186,6 +186,24 @@ class Lwacm:
             raise LwacmError(st, msg)
         return st
 
+    def _after_current(self):
+        """Work enqueued on the library's stream from here on follows torch's current stream."""
+        cur = _torch().cuda.current_stream(self.device)
+        if cur != self.stream:
+            self.stream.wait_stream(cur)
+
+    def _contiguous(self, arrs):
+        """The tensors, contiguous; copies made for that are complete before the library reads them."""
+        for a in arrs:
+            if not a.is_contiguous():
+                break
+        else:
+            return arrs
+        keep = [a.contiguous() for a in arrs]
+        if keep[0].is_cuda:
+            self._after_current()
+        return keep
+
     @property
     def shape(self):
         return (self.ny, self.nx) if self.lattice == D2Q9 else (self.nz, self.ny, self.nx)
@@ -225,7 +243,7 @@ class Lwacm:
             keep = [np.ascontiguousarray(a, dtype=np.float64).reshape(-1) for a in arrs]
             dtype, where = F64, HOST
         else:
-            keep = [a.contiguous() for a in arrs]
+            keep = self._contiguous(arrs)
             dt = keep[0].dtype
             dtype = {torch.float32: F32, torch.float64: F64}[dt]
             where = DEVICE if keep[0].is_cuda else HOST
@@ -255,7 +273,7 @@ class Lwacm:
             dtype, where = F64, HOST
         else:
             torch = _torch()
-            keep = [a.contiguous() for a in arrs]
+            keep = self._contiguous(arrs)
             dtype = {torch.float32: F32, torch.float64: F64}[keep[0].dtype]
             where = DEVICE if keep[0].is_cuda else HOST
         for a in keep:
@@ -278,7 +296,7 @@ class Lwacm:
             keep = np.ascontiguousarray(T, dtype=np.float64).reshape(-1)
             dtype, where = F64, HOST
         else:
-            keep = T.contiguous().reshape(-1)
+            keep, = self._contiguous([T])
             dtype = {torch.float32: F32, torch.float64: F64}[keep.dtype]
             where = DEVICE if keep.is_cuda else HOST
         assert (keep.size if isinstance(keep, np.ndarray) else keep.numel()) == self.n_nodes
@@ -400,6 +418,7 @@ class Lwacm:
         float32 or float64). Returns (grads at the start, dL/dnu)."""
         torch = _torch()
         lam = [t.contiguous() for t in lam]
+        self._after_current()  # lam and the arrays below may come from torch's current stream
         code = F64 if lam[0].dtype == torch.float64 else F32
         outs = [torch.empty_like(t) for t in lam]
         ptrs_in = [t.data_ptr() for t in lam] + [None] * (4 - len(lam))

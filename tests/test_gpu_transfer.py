@@ -119,18 +119,15 @@ def test_force_field_from_memory_of_another_device(lw):
     sim.close()
 
 
-@pytest.mark.parametrize("strided", [False, True])
-def test_fields_outlive_the_call_on_another_stream(lw, strided):
-    """Arrays that are dropped right after set_fields (or copies made of strided ones) are not handed
-    out again while the copy still waits on the context's own stream."""
+def test_fields_outlive_the_call_on_another_stream(lw):
+    """Arrays that are dropped right after set_fields are not handed out again while the copy still
+    waits on the context's own stream."""
     import torch
     n = 64
     st = torch.cuda.Stream()
     sim = lw.Lwacm(9, n, n, 1, 0.02, stream=st)
     g = torch.Generator(device="cuda").manual_seed(84)
     f = [torch.randn(n, n, generator=g, device="cuda") * 0.05 for _ in range(3)]
-    if strided:
-        f = [t.t() for t in f]
     want = [t.cpu().numpy().astype(np.float64) for t in f]
     torch.cuda.synchronize()
     with torch.cuda.stream(st):
@@ -143,3 +140,61 @@ def test_fields_outlive_the_call_on_another_stream(lw, strided):
         assert np.array_equal(a, b)
     assert all(float(t[0, 0]) == 7.0 for t in other)
     sim.close()
+
+
+@pytest.mark.parametrize("call", ["set_fields", "set_force_field", "set_scalar"])
+def test_strided_arrays_on_another_stream(lw, call):
+    """The copies made of strided arrays come from torch's current stream: the context's own stream
+    reads them after it, also when that is busy."""
+    import torch
+    n = 96
+    st = torch.cuda.Stream()
+    sim = lw.Lwacm(9, n, n, 1, 0.02, stream=st, force_field=call == "set_force_field",
+                   scalar_alpha=0.02 if call == "set_scalar" else None)
+    ref = lw.Lwacm(9, n, n, 1, 0.02, force_field=call == "set_force_field",
+                   scalar_alpha=0.02 if call == "set_scalar" else None)
+    g = torch.Generator(device="cuda").manual_seed(85)
+    f = [torch.randn(n, n, generator=g, device="cuda") * 0.05 for _ in range(3)]
+    t = [1e-3 * v.t() for v in f]
+    for s, src in ((ref, [v.contiguous() for v in t]), (sim, t)):
+        s.set_fields(*f)
+        torch.cuda.synchronize()
+        if s is sim:
+            for _ in range(8):  # memory that a copy may get holds other values
+                torch.full((n, n), 7.0, device="cuda")
+            torch.cuda._sleep(50_000_000)  # the copies wait on the current stream
+        if call == "set_fields":
+            s.set_fields(*src)
+        elif call == "set_force_field":
+            s.set_force_field(*src[1:])
+        else:
+            s.set_scalar(src[0])
+        s.step(2)
+        s.sync()
+    for a, b in zip(ref.get_fields(), sim.get_fields()):
+        assert np.array_equal(a, b)
+    if call == "set_scalar":
+        assert np.array_equal(ref.get_scalar(), sim.get_scalar())
+    sim.close()
+    ref.close()
+
+
+def test_backward_on_another_stream(lw):
+    """Seeds that are still being computed on torch's current stream when backward is called."""
+    import torch
+    n = 64
+    out = []
+    for st in (None, torch.cuda.Stream()):
+        sim = lw.Lwacm(9, n, n, 1, 0.02, stream=st)
+        g = torch.Generator(device="cuda").manual_seed(86)
+        f = [torch.randn(n, n, generator=g, device="cuda") * 0.02 for _ in range(6)]
+        torch.cuda.synchronize()
+        sim.set_fields(*f[:3])
+        sim.forward_record(6)
+        sim.sync()
+        torch.cuda._sleep(50_000_000)
+        grads, gnu = sim.backward([v.t() for v in f[3:]])
+        out.append([v.cpu().numpy() for v in grads] + [gnu])
+        sim.close()
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
