@@ -522,6 +522,17 @@ cudaError_t single_dispatch(int shape, const void *in, void *out, const StepPara
     return cudaErrorInvalidValue;
 }
 
+// CTAs of the one-launch form that the GPU holds, and their warps (-1 when it cannot be determined)
+template <int NS, typename T>
+int persistent_grid() {
+    static DevSlots cap;
+    return max_grid(k_batch_rows_persistent<NS, T>, kTile, cap);
+}
+template <int NS, typename T>
+int persistent_room() {
+    const int g = persistent_grid<NS, T>();
+    return g < 1 ? -1 : g * (kTile / 32);
+}
 // D2Q9, shape 0
 template <int NS, typename T>
 cudaError_t rows_t(const void *in, void *out, void *b0, void *b1, const BatchParams &bp, long long nsteps, int parity,
@@ -539,8 +550,7 @@ cudaError_t rows_t(const void *in, void *out, void *b0, void *b1, const BatchPar
         cfg.numAttrs = 1;
         return cudaLaunchKernelEx(&cfg, k_batch_rows<NS, T>, (const T *)in, (T *)out, bp);
     }
-    static DevSlots cap;
-    const int g = max_grid(k_batch_rows_persistent<NS, T>, kTile, cap);
+    const int g = persistent_grid<NS, T>();
     if (g < 1) return cudaErrorNotSupported;
     const long long need = (bp.ntiles + kTile / 32 - 1) / (kTile / 32);
     const long long grid = need < g ? need : g;
@@ -549,15 +559,6 @@ cudaError_t rows_t(const void *in, void *out, void *b0, void *b1, const BatchPar
     void *args[] = {&p0, &p1, &q, &nsteps, &parity};
     return cudaLaunchCooperativeKernel((const void *)k_batch_rows_persistent<NS, T>, dim3((unsigned)grid), dim3(kTile),
                                        args, 0, st);
-}
-// warps of the kernel that the GPU holds (-1 when it cannot be determined)
-template <int NS, typename T>
-int rows_room(bool one_launch) {
-    static DevSlots cap[2];
-    const int w = one_launch ? kTile / 32 : rows_warps(NS);
-    const int g = one_launch ? max_grid(k_batch_rows_persistent<NS, T>, 32 * w, cap[1])
-                             : max_grid(k_batch_rows<NS, T>, 32 * w, cap[0]);
-    return g < 1 ? -1 : g * w;
 }
 cudaError_t rows_storage(int storage, const void *in, void *out, void *b0, void *b1, const BatchParams &bp,
                          long long nsteps, int parity, bool persistent, cudaStream_t st) {
@@ -608,27 +609,28 @@ cudaError_t runs_t(int Q, void *b0, void *b1, const BatchParams &bp, long long n
 
 int batch_tile() { return kTile; }
 int batch_rows_strip() { return rows2::kHalf; }
-// The cut of one domain (rows2.cuh) over the whole ensemble's strips, for the warps the GPU holds of
-// the kernel that runs (28 or 32 a SM of the one-strip form with a launch a step, 23 of the other,
-// 24 and 16 in one launch for all; `device`: asked of the current one, else those of a GB300). 256
-// domains of 32 to 512 nodes a side: 17 rows 37.7 us a step, 4 rows 46.3, 64 rows 45.2, one strip a
-// warp 42.4 at best. The one-launch form cut for its own room, in place of the other form's: 20
-// domains of 10 x 200 4.1 us a step against 5.7, 300 of 10 x 64 7.2 against 9.3, 100 of 300^2 54.9
-// against 63.1.
+// The cut of one domain (rows2.cuh) over the whole ensemble's strips, for the warps the GPU holds
+// of the kernel that runs. A launch a step: 28 a SM of the one-strip form and 23 of the other, the
+// figures the cut was measured with (256 domains of 32 to 512 nodes a side: 13 rows 39.0 us a step,
+// 15 rows, for the 20 that the occupancy gives, 39.5, 4 rows 46.3, 64 rows 45.2, one strip a warp
+// 42.4 at best). One launch for all: what the occupancy gives, since its items wait for one another
+// at the barrier (20 domains of 10 x 200 4.1 us a step, cut for the other form's room 5.7, 300 of 10
+// x 64 7.2 and 9.3, 100 of 300^2 54.9 and 63.1). device: for the current device, else a GB300.
 void batch_rows_cut(const BatchDomain *doms, int n, int storage, bool one_launch, bool device, int *ns, int *rows) {
     long long w1 = 0, w2 = 0;
     for (int b = 0; b < n; ++b) {
         w1 += (long long)((doms[b].nx - 1) / rows2::kHalf + 1) * doms[b].ny;
         w2 += (long long)((doms[b].nx - 1) / (2 * rows2::kHalf) + 1) * doms[b].ny;
     }
-    long long r1 = (one_launch ? 24 : 28) * 152, r2 = (one_launch ? 16 : 23) * 152;
-    if (device) {
-        const int d1 = storage == STORE_F32    ? rows_room<1, float>(one_launch)
-                       : storage == STORE_BF16 ? rows_room<1, __nv_bfloat16>(one_launch)
-                                               : rows_room<1, __half>(one_launch);
-        const int d2 = storage == STORE_F32    ? rows_room<2, float>(one_launch)
-                       : storage == STORE_BF16 ? rows_room<2, __nv_bfloat16>(one_launch)
-                                               : rows_room<2, __half>(one_launch);
+    const long long sms = device ? device_sms() : 152;
+    long long r1 = (one_launch ? 24 : 28) * sms, r2 = (one_launch ? 16 : 23) * sms;
+    if (device && one_launch) {
+        const int d1 = storage == STORE_F32    ? persistent_room<1, float>()
+                       : storage == STORE_BF16 ? persistent_room<1, __nv_bfloat16>()
+                                               : persistent_room<1, __half>();
+        const int d2 = storage == STORE_F32    ? persistent_room<2, float>()
+                       : storage == STORE_BF16 ? persistent_room<2, __nv_bfloat16>()
+                                               : persistent_room<2, __half>();
         if (d1 > 0 && d2 > 0) r1 = d1, r2 = d2;
     }
     const rows2::Cut c = rows2::cut_rows(w1, w2, r1, r2);
