@@ -639,8 +639,9 @@ def run_gpu(args):
     return 0
 
 
-def run_case(name, steps):
-    """One variant workload, stepped without timing (a target for profilers)."""
+def run_case(name, steps, kernel=0, tile=None):
+    """One variant workload, stepped without timing (a target for profilers); kernel and tile:
+    LWACM_OPT_KERNEL and LWACM_OPT_BATCH_TILE where a case has a choice."""
     import torch
     from paper_1111_2142_gb300 import inputs
     from paper_1111_2142_gb300 import lwacm as lw
@@ -653,14 +654,16 @@ def run_case(name, steps):
         lam = [torch.zeros((n3, n3, n3), device="cuda")] + [
             torch.tensor(a, dtype=torch.float32, device="cuda") for a in fa[1:]]
         sim.backward(lam)
-    elif name == "ensemble":  # 256 D2Q9 domains (seed 1), 2D tiles 30x14
+    elif name == "ensemble":  # 256 D2Q9 domains (seed 1), 2D tiles 30x14 unless --tile says otherwise
         doms = inputs.ensemble_2d(256, seed=1)
-        sim = lw.LwacmBatch(lw.D2Q9, [(d["nx"], d["ny"]) for d in doms], [d["nu"] for d in doms], tile=2)
+        sim = lw.LwacmBatch(lw.D2Q9, [(d["nx"], d["ny"]) for d in doms], [d["nu"] for d in doms],
+                            tile=2 if tile is None else tile)
         sim.set_domains([(d["d"], d["ux"], d["uy"]) for d in doms])
         sim.step(steps)
     elif name == "cavity":  # D2Q9 1024^2 lid-driven cavity, Re 1000, from rest
         z = torch.zeros((1024, 1024), dtype=torch.float32, device="cuda")
         sim = lw.Lwacm(lw.D2Q9, 1024, 1024, 1, 0.1024, lw.CAVITY, lid=(0.1, 0.0))
+        sim.set_option(lw.OPT_BATCH_TILE, tile or 0)
         sim.set_fields(z, z, z)
         sim.step(steps)
     elif name == "cavity3d":  # D3Q19 256^3 diagonally driven cavity from rest (half-row kernel + walls)
@@ -679,14 +682,30 @@ def run_case(name, steps):
         sim.set_option(lw.OPT_NU_P, 0.05)
         sim.set_fields(*inputs.tgv3d(256, u0=U0))
         sim.step(steps)
-    elif name == "segments":  # D3Q19 384 x 256 x 128 Taylor-Green (marching warps)
-        sim = lw.Lwacm(lw.D3Q19, 384, 256, 128, NU)
+    elif name == "segments":  # D3Q19 384 x 256 x 128 Taylor-Green (marching warps; kernel 5: half-row segments)
+        sim = lw.Lwacm(lw.D3Q19, 384, 256, 128, NU, kernel=kernel)
         sim.set_fields(*inputs.tgv3d(384, u0=U0, ny=256, nz=128))
         sim.step(steps)
     elif name == "bulk2d":  # D2Q9 4096^2 bulk-viscosity variant, gamma 0.4 (marching warps)
         sim = lw.Lwacm(lw.D2Q9, 4096, 4096, 1, 0.01, bulk_gamma=0.4)
+        sim.set_option(lw.OPT_BATCH_TILE, tile or 0)
         sim.set_fields(*inputs.gtg_state(4096, 0.0))
         sim.step(steps)
+    elif name == "periodic2d":  # D2Q9 4096^2, plain scheme
+        sim = lw.Lwacm(lw.D2Q9, 4096, 4096, 1, 0.01)
+        sim.set_option(lw.OPT_BATCH_TILE, tile or 0)
+        sim.set_fields(*inputs.gtg_state(4096, 0.0))
+        sim.step(steps)
+    elif name == "small2d":  # D2Q9 128^2, bulk viscosity and omega_p: the steps in one launch of a cluster
+        sim = lw.Lwacm(lw.D2Q9, 128, 128, 1, 5.12e-4, bulk_gamma=0.4)
+        sim.set_option(lw.OPT_NU_P, 170 * 5.12e-4)
+        sim.set_fields(*inputs.tgv2d(128, u0=0.04))
+        sim.step(steps)
+    elif name == "diagnostics":  # global quantities of a D3Q19 256^3 state, `steps` calls
+        sim = lw.Lwacm(lw.D3Q19, 256, 256, 256, NU)
+        sim.set_fields(*inputs.tgv3d(256, u0=U0))
+        for _ in range(steps):
+            sim.diagnostics()
     else:
         raise SystemExit(f"unknown case {name}")
     sim.sync()
@@ -708,8 +727,9 @@ def main():
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--no-variants", action="store_true")
     ap.add_argument("--profile-case", choices=["adjoint", "ensemble", "cavity", "cavity3d", "bulk2d", "scalar",
-                                               "segments", "nu_p3d"],
+                                               "segments", "nu_p3d", "periodic2d", "small2d", "diagnostics"],
                     help="run one variant workload for --steps steps without timing (for profilers)")
+    ap.add_argument("--tile", type=int, default=None, help="LWACM_OPT_BATCH_TILE of a --profile-case")
     args = ap.parse_args()
     if args.warmup < 3:
         args.warmup = 3
@@ -718,7 +738,7 @@ def main():
     import __graft_entry__
     __graft_entry__.build()
     if args.profile_case:
-        return run_case(args.profile_case, args.steps)
+        return run_case(args.profile_case, args.steps, args.kernel, args.tile)
     return run_gpu(args)
 
 

@@ -10,7 +10,7 @@
 // ACM2.0b(a)) and hands them on without shared memory or a barrier (stream, Eq.
 // ACM2.0b(b)): along x by warp shuffles, along y through the sums of three rows kept in
 // registers, of which the oldest is complete once the next row has been read
-// (post-combine, Eq. ACM2.0b(c)). The loads of the row after next are in flight
+// (post-combine, Eq. ACM2.0b(c)). The loads of the next four rows are in flight
 // meanwhile.
 //
 // What bounds it, FP32 periodic: at 8192^2 memory (262 us a step, 6.1 TB/s, 91% of a copy's

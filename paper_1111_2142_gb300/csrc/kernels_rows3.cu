@@ -200,8 +200,7 @@ struct March3 {
     }
     template <int MODE>
     __device__ __forceinline__ void to_rows(const Node &n, Send &up, Send &dn) const {
-        constexpr bool OWN = MODE == START || MODE == MID, DOWN = MODE == MID || MODE == LAST, UP = MODE != LAST;
-        if (OWN) {
+        if (MODE == START || MODE == MID) {
             F2 yp, ym, pp, mm, pm, mp;
             pair(n, n.v, false, yp, ym);
             pair(n, add(n.u, n.v), true, pp, mm);  // (1,1,0) (-1,-1,0)
@@ -215,8 +214,6 @@ struct March3 {
         }
         pair(n, add(n.v, n.w), true, up.p, dn.m);  // (0,1,1) (0,-1,-1)
         pair(n, sub(n.v, n.w), true, up.m, dn.p);  // (0,1,-1) (0,-1,1)
-        (void)DOWN;
-        (void)UP;
     }
     // rows 0 (up) and 5 (down, its v negated): what they send to the tile
     template <int MODE>

@@ -313,16 +313,17 @@ void build_rows2(lwacm_ctx *c, int mode, bool device) {
 
 // upload the tile table of the current shape and launch form (host tables are pageable: synchronise)
 lwacm_status upload_tiles(lwacm_ctx *c) {
-    if (!c->rows2.empty()) {
-        try {  // cut for this device, or as the workspace was sized
+    try {
+        if (c->batch_shape > 0) {
+            build_tiles2(c, c->batch_shape, c->tiles2);
+        } else if (!c->rows2.empty()) {  // cut for this device, or as the workspace was sized
             build_rows2(c, c->batch_mode, true);
             if (sizeof(BatchRows) * c->rows2.size() > c->tiles_cap) build_rows2(c, c->batch_mode, false);
-        } catch (...) {
-            return fail(c, LWACM_E_NOMEM, "table of strips");
         }
+    } catch (...) {
+        return fail(c, LWACM_E_NOMEM, "tile table");
     }
     if (c->batch_shape > 0) {
-        build_tiles2(c, c->batch_shape, c->tiles2);
         CK(c, cudaMemcpyAsync(c->ws + c->off_tiles, c->tiles2.data(), sizeof(BatchTile2) * c->tiles2.size(),
                               cudaMemcpyHostToDevice, c->stream),
            "tile table");
