@@ -613,9 +613,11 @@ int batch_rows_strip() { return rows2::kHalf; }
 // of the kernel that runs. A launch a step: 28 a SM of the one-strip form and 23 of the other, the
 // figures the cut was measured with (256 domains of 32 to 512 nodes a side: 13 rows 39.0 us a step,
 // 15 rows, for the 20 that the occupancy gives, 39.5, 4 rows 46.3, 64 rows 45.2, one strip a warp
-// 42.4 at best). One launch for all: what the occupancy gives, since its items wait for one another
-// at the barrier (20 domains of 10 x 200 4.1 us a step, cut for the other form's room 5.7, 300 of 10
-// x 64 7.2 and 9.3, 100 of 300^2 54.9 and 63.1). device: for the current device, else a GB300.
+// 42.4 at best). One launch for all: what the occupancy gives, and the rows that waste least of the
+// whole rounds of items that fit between two barriers (cut for the other form's room / for its own /
+// for whole rounds: 20 domains of 10 x 200 5.7 / 4.1 / 4.1 us a step, 300 of 33 x 64 11.3 / 8.8 / 8.8,
+// 100 of 300^2 63.1 / 55.4 / 55.4, the 256 domains 53.8 / 55.7 / 49.3). device: for the current
+// device, else a GB300.
 void batch_rows_cut(const BatchDomain *doms, int n, int storage, bool one_launch, bool device, int *ns, int *rows) {
     long long w1 = 0, w2 = 0;
     for (int b = 0; b < n; ++b) {
@@ -633,7 +635,18 @@ void batch_rows_cut(const BatchDomain *doms, int n, int storage, bool one_launch
                                                : persistent_room<2, __half>();
         if (d1 > 0 && d2 > 0) r1 = d1, r2 = d2;
     }
-    const rows2::Cut c = rows2::cut_rows(w1, w2, r1, r2);
+    rows2::Cut c = rows2::cut_rows(w1, w2, r1, r2);
+    if (one_launch) {  // whole rounds of items between two barriers: the rows that take the fewest row times
+        const long long room = c.ns == 1 ? r1 : r2;
+        long long least = -1;
+        for (int h = 1; h <= 32; ++h) {
+            long long items = 0;
+            for (int b = 0; b < n; ++b)
+                items += (long long)((doms[b].nx - 1) / (c.ns * rows2::kHalf) + 1) * ((doms[b].ny - 1) / h + 1);
+            const long long cost = ((items - 1) / room + 1) * (2 * h + 3);
+            if (least < 0 || cost < least) least = cost, c.rows = h;
+        }
+    }
     *ns = c.ns;
     *rows = c.rows;
 }
