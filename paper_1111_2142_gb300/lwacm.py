@@ -168,8 +168,9 @@ class Lwacm:
             self.device = torch.device(device if device is not None else "cuda")
             self.workspace = torch.empty(nbytes.value, dtype=torch.uint8, device=self.device)
             self.stream = stream if stream is not None else torch.cuda.current_stream(self.device)
+            self._raw_stream, self._device_index = self.stream.cuda_stream, self.workspace.device.index
             self._check(lib.lwacm_bind(h, self.workspace.data_ptr(), nbytes.value,
-                                       ctypes.c_void_p(self.stream.cuda_stream)))
+                                       ctypes.c_void_p(self._raw_stream)))
             if kernel:  # explicit kernels are checked against the bound device
                 self._check(lib.lwacm_set_option(h, OPT_KERNEL, float(kernel)))
         except Exception:
@@ -256,9 +257,10 @@ class Lwacm:
             self.sync()
             self._hold = None
         else:
-            for a in keep:  # the copy runs on the library's stream
-                if a.is_cuda:
-                    a.record_stream(self.stream)
+            if torch._C._cuda_getCurrentRawStream(self._device_index) != self._raw_stream:
+                for a in keep:  # the copy runs on the library's stream, the caller's work elsewhere
+                    if a.is_cuda:
+                        a.record_stream(self.stream)
 
     def set_force_field(self, gx, gy, gz=None):
         """Per-node acceleration g(x) of Eq. force for the following steps (needs
