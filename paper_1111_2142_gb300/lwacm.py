@@ -187,11 +187,14 @@ class Lwacm:
             raise LwacmError(st, msg)
         return st
 
+    def _elsewhere(self):
+        """Whether torch's current stream is not the library's (a stream object for it takes 10 us)."""
+        return _torch()._C._cuda_getCurrentRawStream(self._device_index) != self._raw_stream
+
     def _after_current(self):
         """Work enqueued on the library's stream from here on follows torch's current stream."""
-        cur = _torch().cuda.current_stream(self.device)
-        if cur != self.stream:
-            self.stream.wait_stream(cur)
+        if self._elsewhere():
+            self.stream.wait_stream(_torch().cuda.current_stream(self.device))
 
     def _contiguous(self, arrs):
         """The tensors, contiguous; copies made for that are complete before the library reads them."""
@@ -240,7 +243,7 @@ class Lwacm:
         (CUDA or host, float32/float64)."""
         arrs = [d, ux, uy] + ([uz] if self.lattice == D3Q19 else [])
         torch = _torch()
-        if all(isinstance(a, np.ndarray) for a in arrs):
+        if isinstance(arrs[0], np.ndarray) and all(isinstance(a, np.ndarray) for a in arrs):
             keep = [np.ascontiguousarray(a, dtype=np.float64).reshape(-1) for a in arrs]
             dtype, where = F64, HOST
         else:
@@ -257,7 +260,7 @@ class Lwacm:
             self.sync()
             self._hold = None
         else:
-            if torch._C._cuda_getCurrentRawStream(self._device_index) != self._raw_stream:
+            if self._elsewhere():
                 for a in keep:  # the copy runs on the library's stream, the caller's work elsewhere
                     if a.is_cuda:
                         a.record_stream(self.stream)
@@ -270,7 +273,7 @@ class Lwacm:
             self._check(self._lib.lwacm_set_force_field(self._h, None, None, None, F32, DEVICE))
             return
         arrs = [gx, gy] + ([gz] if self.lattice == D3Q19 else [])
-        if all(isinstance(a, np.ndarray) for a in arrs):
+        if isinstance(arrs[0], np.ndarray) and all(isinstance(a, np.ndarray) for a in arrs):
             keep = [np.ascontiguousarray(a, dtype=np.float64).reshape(-1) for a in arrs]
             dtype, where = F64, HOST
         else:
