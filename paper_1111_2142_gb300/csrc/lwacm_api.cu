@@ -79,10 +79,12 @@ struct lwacm_ctx {
     int nbatch = 0;
     std::vector<BatchDomain> doms;
     // shape 0: strips and runs of rows (D2Q9) or 1D tiles (D3Q19, narrow D2Q9 domains; rows2 is empty),
-    // the same in both launch forms, which give the same fields bit for bit
-    std::vector<BatchRows> rows2;
+    // the same in both launch forms, which give the same fields bit for bit. The strips are cut for
+    // each form; the workspace holds both tables, so that a graph of one outlives a change of form
+    std::vector<BatchRows> rows2[2];
     std::vector<BatchTile> tiles;
-    int rows_ns = 1;                 // strips per warp of rows2
+    int rows_ns[2] = {1, 1};         // strips per warp of rows2
+    size_t rows_cap[2] = {0, 0};     // bytes reserved for each table, the second after the first
     std::vector<BatchTile2> tiles2;  // 2D tiles of the current shape (shape > 0)
     int batch_shape = 0;
     size_t tiles_cap = 0;  // table bytes reserved in the workspace (largest over the shapes)
@@ -220,7 +222,7 @@ bool choose_kernel(lwacm_ctx *c) {
             {"batch_persistent", "batch_tiles30x6_persistent", "batch_tiles30x14_persistent",
              "batch_tiles62x6_persistent", "batch_tiles30x30_persistent", "batch_tiles62x14_persistent",
              "batch_tiles126x6_persistent", "batch_rows_persistent"}};
-        c->kname = names[c->batch_mode ? 1 : 0][c->batch_shape == 0 && !c->rows2.empty() ? 7 : c->batch_shape];
+        c->kname = names[c->batch_mode ? 1 : 0][c->batch_shape == 0 && !c->rows2[0].empty() ? 7 : c->batch_shape];
         return c->kernel_opt == 0 || c->kernel_opt == 1;
     }
     const StepParams p = params(c);
@@ -292,9 +294,9 @@ void build_tiles2(const lwacm_ctx *c, int k, std::vector<BatchTile2> &out) {
 // current device
 void build_rows2(lwacm_ctx *c, int mode, bool device) {
     int rows = 1;
-    batch_rows_cut(c->doms.data(), c->nbatch, c->storage, mode == 1, device, &c->rows_ns, &rows);
-    const int width = c->rows_ns * batch_rows_strip();
-    c->rows2.clear();
+    batch_rows_cut(c->doms.data(), c->nbatch, c->storage, mode == 1, device, &c->rows_ns[mode], &rows);
+    const int width = c->rows_ns[mode] * batch_rows_strip();
+    c->rows2[mode].clear();
     for (const BatchDomain &d : c->doms)
         for (int y = 0; y < d.ny; y += rows)
             for (int x = 0; x < d.nx; x += width) {
@@ -307,18 +309,19 @@ void build_rows2(lwacm_ctx *c, int mode, bool device) {
                 r.yb = d.ny - y > rows ? y + rows : d.ny;
                 r.s = d.s;
                 r.a = d.a;
-                c->rows2.push_back(r);
+                c->rows2[mode].push_back(r);
             }
 }
 
-// upload the tile table of the current shape and launch form (host tables are pageable: synchronise)
+// upload the tile table of the current shape (host tables are pageable: synchronise)
 lwacm_status upload_tiles(lwacm_ctx *c) {
     try {
         if (c->batch_shape > 0) {
             build_tiles2(c, c->batch_shape, c->tiles2);
-        } else if (!c->rows2.empty()) {  // cut for this device, or as the workspace was sized
-            build_rows2(c, c->batch_mode, true);
-            if (sizeof(BatchRows) * c->rows2.size() > c->tiles_cap) build_rows2(c, c->batch_mode, false);
+        }
+        for (int m = 0; m < 2 && c->batch_shape == 0 && !c->rows2[m].empty(); ++m) {
+            build_rows2(c, m, true);  // cut for this device, or as the workspace was sized
+            if (sizeof(BatchRows) * c->rows2[m].size() > c->rows_cap[m]) build_rows2(c, m, false);
         }
     } catch (...) {
         return fail(c, LWACM_E_NOMEM, "tile table");
@@ -327,10 +330,11 @@ lwacm_status upload_tiles(lwacm_ctx *c) {
         CK(c, cudaMemcpyAsync(c->ws + c->off_tiles, c->tiles2.data(), sizeof(BatchTile2) * c->tiles2.size(),
                               cudaMemcpyHostToDevice, c->stream),
            "tile table");
-    } else if (!c->rows2.empty()) {
-        CK(c, cudaMemcpyAsync(c->ws + c->off_tiles, c->rows2.data(), sizeof(BatchRows) * c->rows2.size(),
-                              cudaMemcpyHostToDevice, c->stream),
-           "tile table");
+    } else if (!c->rows2[0].empty()) {
+        for (int m = 0; m < 2; ++m)
+            CK(c, cudaMemcpyAsync(c->ws + c->off_tiles + m * c->rows_cap[0], c->rows2[m].data(),
+                                  sizeof(BatchRows) * c->rows2[m].size(), cudaMemcpyHostToDevice, c->stream),
+               "tile table");
     } else {
         CK(c, cudaMemcpyAsync(c->ws + c->off_tiles, c->tiles.data(), sizeof(BatchTile) * c->tiles.size(),
                               cudaMemcpyHostToDevice, c->stream),
@@ -343,13 +347,14 @@ lwacm_status upload_tiles(lwacm_ctx *c) {
 BatchParams batch_params(lwacm_ctx *c) {
     BatchParams bp;
     bp.doms = (const BatchDomain *)(c->ws + c->off_doms);
-    const bool rows = !c->rows2.empty();
+    const std::vector<BatchRows> &r = c->rows2[c->batch_mode];
+    const bool rows = !r.empty();
     bp.tiles = (const BatchTile *)(c->ws + c->off_tiles);
     bp.tiles2 = (const BatchTile2 *)(c->ws + c->off_tiles);
-    bp.rows2 = rows ? (const BatchRows *)(c->ws + c->off_tiles) : nullptr;
-    bp.ns = c->rows_ns;
+    bp.rows2 = rows ? (const BatchRows *)(c->ws + c->off_tiles + c->batch_mode * c->rows_cap[0]) : nullptr;
+    bp.ns = c->rows_ns[c->batch_mode];
     bp.shape = c->batch_shape;
-    bp.ntiles = (long long)(c->batch_shape > 0 ? c->tiles2.size() : (rows ? c->rows2.size() : c->tiles.size()));
+    bp.ntiles = (long long)(c->batch_shape > 0 ? c->tiles2.size() : (rows ? r.size() : c->tiles.size()));
     bp.fstride = c->Nal;
     bp.bar_count = (unsigned *)(c->ws + c->off_bar);
     bp.bar_gen = bp.bar_count + 1;
@@ -656,9 +661,9 @@ lwacm_status lwacm_batch_create(int lattice, int n, const int *nx, const int *ny
             off += d.n;
         }
         const bool rows = lattice == LWACM_D2Q9 && batch_rows_pays(c->doms.data(), n);
-        for (int m = 1; rows && m >= 0; --m) {
+        for (int m = 0; rows && m < 2; ++m) {
             build_rows2(c, m, false);
-            c->tiles_cap = std::max(c->tiles_cap, sizeof(BatchRows) * c->rows2.size());
+            c->rows_cap[m] = align_up(sizeof(BatchRows) * c->rows2[m].size(), kAlign);
         }
         for (int b = 0; b < n && !rows; ++b)
             for (long long t = 0; t < c->doms[b].n; t += tile) {
@@ -673,7 +678,7 @@ lwacm_status lwacm_batch_create(int lattice, int n, const int *nx, const int *ny
         return LWACM_E_NOMEM;
     }
     try {
-        c->tiles_cap = std::max(c->tiles_cap, sizeof(BatchTile) * c->tiles.size());
+        c->tiles_cap = std::max(c->rows_cap[0] + c->rows_cap[1], sizeof(BatchTile) * c->tiles.size());
         if (lattice == LWACM_D2Q9) {
             std::vector<BatchTile2> t2;
             for (int k = 1; k < batch_shapes(); ++k) {
@@ -758,12 +763,7 @@ lwacm_status lwacm_set_option(lwacm_ctx *c, int key, double v) {
             const int m = (int)v;
             if (m != 0 && m != 1) return fail(c, LWACM_E_ARG, "batch mode must be 0 or 1");
             if (!c->nbatch) return fail(c, LWACM_E_STATE, "not a batched context");
-            const bool other = m != c->batch_mode;
             c->batch_mode = m;
-            if (other && c->bound && !c->rows2.empty() && c->batch_shape == 0) {
-                const lwacm_status ts = upload_tiles(c);
-                if (ts != LWACM_OK) return ts;
-            }
             break;
         }
         case LWACM_OPT_SCALAR_ALPHA: {

@@ -221,3 +221,31 @@ def test_narrow_ensembles(lw, dims, rows, storage):
                 tol = 1.05 * 2.0 ** -8 * np.abs(r) + 8 * 2.0 ** -24 * 0.04 if storage else 4e-7
                 assert np.all(np.abs(g - r) <= tol)
     sim.close()
+
+
+def test_a_graph_of_one_launch_form_outlives_a_change_to_the_other(lw):
+    """Steps captured with a launch a step replay the same after the context has run the one-launch
+    form, whose strips are cut otherwise."""
+    import torch
+    dims, nus = [(10, 200)] * 20 + [(70, 31)], [0.01 + 0.001 * b for b in range(21)]
+    fields = [inputs.smooth_random((h, w), seed=950 + b, u_amp=0.04, d_amp=0.01) for b, (w, h) in enumerate(dims)]
+    sim = lw.LwacmBatch(9, dims, nus, graph_chunk=0, stream=torch.cuda.Stream())
+    assert sim.kernel_name == "batch_rows_step"
+    sim.set_domains(fields)
+    sim.step(2)
+    want = sim.get_domains()
+    sim.set_domains(fields)
+    sim.sync()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=sim.stream):
+        sim.step(2)
+    sim.set_option(lw.OPT_BATCH_MODE, 1)
+    sim.set_domains(fields)
+    sim.step(2)
+    assert all(np.array_equal(a, b) for x, y in zip(sim.get_domains(), want) for a, b in zip(x, y))
+    sim.set_domains(fields)
+    with torch.cuda.stream(sim.stream):
+        g.replay()
+    sim.sync()
+    assert all(np.array_equal(a, b) for x, y in zip(sim.get_domains(), want) for a, b in zip(x, y))
+    sim.close()
