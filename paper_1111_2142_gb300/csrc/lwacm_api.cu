@@ -373,8 +373,9 @@ cudaError_t step_between(lwacm_ctx *c, const void *in, void *out, cudaStream_t s
     if (c->kernel == 5 && p.sdelta != 0.f) e = launch_nup_sum(c->storage, in, p.nup_p, p, st);
     if (e != cudaSuccess) return e;
     // Recorded runs and their recomputation stay on the half-row, 2D-tile and gather kernels: dL/dnu
-    // is a sum that may cancel, and the marching kernels' other order of additions moved it by more
-    // than 2e-5 in one of five random runs
+    // is a sum that may cancel, and the marching kernels' other order of additions moves it by more
+    // than 2e-5 in one of six random runs (60 runs against FP64: the median error the same, 7.7e-7 and
+    // 8.1e-7, but in three of them more than 1.5 times as large)
     const bool rec = c->recording;
     const bool march = c->march && !rec;
     e = march            ? launch_step_rows3d(c->storage, in, out, pf, st)
